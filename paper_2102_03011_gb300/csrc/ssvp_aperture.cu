@@ -85,12 +85,12 @@ __global__ void __launch_bounds__(kApThreads, 4) aperture_kernel(const GatherArg
                 continue;
             }
             const float4 q0 = g[0], q1 = g[1], q2 = g[2], q3 = g[3], q4 = g[4];
-            const df m0 = df_add_f({q0.x, q0.w}, __fmaf_rn(q1.z, du, __fmul_rn(q1.w, dv)));
-            const df m1 = df_add_f({q0.y, q1.x}, __fmaf_rn(q2.x, du, __fmul_rn(q2.y, dv)));
-            const df m2 = df_add_f({q0.z, q1.y}, __fmaf_rn(q2.z, du, __fmul_rn(q2.w, dv)));
-            const df w0 = df_add(df_mul_f(m0, dref), {q3.x, q3.w});
-            const df w1 = df_add(df_mul_f(m1, dref), {q3.y, q4.x});
-            const df w2 = df_add(df_mul_f(m2, dref), {q3.z, q4.y});
+            const df m0 = df_add_f({q0.x, q0.z}, __fmaf_rn(q1.x, du, __fmul_rn(q1.z, dv)));
+            const df m1 = df_add_f({q0.y, q0.w}, __fmaf_rn(q1.y, du, __fmul_rn(q1.w, dv)));
+            const df m2 = df_add_f({q3.x, q3.y}, __fmaf_rn(q3.z, du, __fmul_rn(q3.w, dv)));
+            const df w0 = df_add(df_mul_f(m0, dref), {q2.x, q2.z});
+            const df w1 = df_add(df_mul_f(m1, dref), {q2.y, q2.w});
+            const df w2 = df_add(df_mul_f(m2, dref), {q4.x, q4.y});
             if (!(w2.hi > 1e-6f * dref) || !(m2.hi > 0.0f)) {
                 if (DEBUG && rec) rec[0] = 0;
                 continue;
@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(kApThreads, 4) aperture_kernel(const GatherArg
             float mnx = 3.0e38f, mny = 3.0e38f, mxx = -3.0e38f, mxy = -3.0e38f, sx = 0.0f, sy = 0.0f;
             bool behind = false;
             {
-                const float c0x = fxO * q1.z, c0y = fxO * q2.x, c0z = fxO * q2.z;
-                const float c1x = fyO * q1.w, c1y = fyO * q2.y, c1z = fyO * q2.w;
+                const float c0x = fxO * q1.x, c0y = fxO * q1.y, c0z = fxO * q3.z;
+                const float c1x = fyO * q1.z, c1y = fyO * q1.w, c1z = fyO * q3.w;
                 for (int i = 0; i < a.lens_n; ++i) {
                     const float lx = a.aperture * a.lens_xy[2 * i] * s_seed, ly = a.aperture * a.lens_xy[2 * i + 1] * s_seed;
                     const float wx = fmaf(lx, c0x, fmaf(ly, c1x, w0.hi));

@@ -72,6 +72,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+constexpr unsigned kMagic = 0x4b000000u;  // bits of 2^23: n | kMagic is the float 2^23 + n for n < 2^23
 // exact float of a small non-negative integer (< 2^23) without a conversion instruction
 __device__ __forceinline__ float small_float(int v) { return __int_as_float(0x4b000000 | v) - 8388608.0f; }
 
@@ -134,17 +135,34 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
     return d;
 }
 
+// One window sample as two pairs, (r, g) and (b, depth): for FP32 colour the record's halves as loaded
+template <int CFMT>
+__device__ __forceinline__ void load_record(const float *dwin, const void *cwin, int idx, f32x2 &rg, f32x2 &bz) {
+    if (CFMT == 0) {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(cwin) + idx);
+        rg = v.x;
+        bz = v.y;
+    } else {
+        float d;
+        float3 c;
+        load_sample<1>(dwin, cwin, idx, d, c);
+        rg = f2_pack(c.x, c.y);
+        bz = f2_pack(c.z, d);
+    }
+}
+
 __device__ __forceinline__ f32x2 f2_abs(f32x2 a) { return a & 0x7fffffff7fffffffull; }
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kSlotVec = 6;  // float4 words of per-slot geometry in shared memory
 
-// Shared per-slot geometry (6 x float4):
-//  q0 = mb_hi0 mb_hi1 mb_hi2 mb_lo0   (mb = M (u0, v0, 1) of the CTA's first pixel, double-float)
-//  q1 = mb_lo1 mb_lo2 M00 M01
-//  q2 = M10 M11 M20 M21
-//  q3 = e_hi0 e_hi1 e_hi2 e_lo0
-//  q4 = e_lo1 e_lo2 ifx ify
+// Shared per-slot geometry (6 x float4), the x and y rows side by side so that packed FP32x2
+// operations take them as they are:
+//  q0 = mb_hi0 mb_hi1 mb_lo0 mb_lo1   (mb = M (u0, v0, 1) of the CTA's first pixel, double-float)
+//  q1 = M00 M10 M01 M11
+//  q2 = e_hi0 e_hi1 e_lo0 e_lo1
+//  q3 = mb_hi2 mb_lo2 M20 M21
+//  q4 = e_hi2 e_lo2 ifx ify
 //  q5 = cx cy beta*log2e J(bits)
 __device__ void build_slot(const PairGeom &g, float u0, float v0, float4 *dst) {
     df mb[3];
@@ -154,11 +172,11 @@ __device__ void build_slot(const PairGeom &g, float u0, float v0, float4 *dst) {
         t = df_add(t, df_mul_f({g.M_hi[3 * r + 1], g.M_lo[3 * r + 1]}, v0));
         mb[r] = df_add(t, {g.M_hi[3 * r + 2], g.M_lo[3 * r + 2]});
     }
-    dst[0] = make_float4(mb[0].hi, mb[1].hi, mb[2].hi, mb[0].lo);
-    dst[1] = make_float4(mb[1].lo, mb[2].lo, g.M_hi[0], g.M_hi[1]);
-    dst[2] = make_float4(g.M_hi[3], g.M_hi[4], g.M_hi[6], g.M_hi[7]);
-    dst[3] = make_float4(g.e_hi[0], g.e_hi[1], g.e_hi[2], g.e_lo[0]);
-    dst[4] = make_float4(g.e_lo[1], g.e_lo[2], g.ifx, g.ify);
+    dst[0] = make_float4(mb[0].hi, mb[1].hi, mb[0].lo, mb[1].lo);
+    dst[1] = make_float4(g.M_hi[0], g.M_hi[3], g.M_hi[1], g.M_hi[4]);
+    dst[2] = make_float4(g.e_hi[0], g.e_hi[1], g.e_lo[0], g.e_lo[1]);
+    dst[3] = make_float4(mb[2].hi, mb[2].lo, g.M_hi[6], g.M_hi[7]);
+    dst[4] = make_float4(g.e_hi[2], g.e_lo[2], g.ifx, g.ify);
     dst[5] = make_float4(g.cx, g.cy, g.beta * kLog2e, __int_as_float(g.J));
 }
 

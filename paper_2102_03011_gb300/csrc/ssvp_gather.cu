@@ -14,12 +14,24 @@
 //     Y_q - y_ref = ((d_q - z') (q_x - c_x) + z' (q_x - u')) / f_x, ... , d_q - z'
 // so the FP32 error of the distance is ~1e-7 of the radius rather than ~1e-7 of the depth.
 //
-// Accepted candidates are recorded in a per-thread bit mask during the test loop and filtered
-// afterwards by iterating the set bits, so a warp pays for the filter arithmetic only as often
-// as its busiest lane accepts (warp-level compaction of the accepted samples).
+// Two loops per (pixel, J).  The test loop runs over the k x k window two columns at a time (aligned
+// 8-byte loads, packed FP32x2) and only decides which candidates can be samples: by the depth part of
+// the distance alone, or, where the radius is small against the window, by all of it (see lateral).
+// Its threshold is widened so that it keeps every sample; the sign of each result is shifted into a bit
+// mask.  The filter loop takes the mask's bits, three (FP32 colour) or two at a time so that their
+// loads overlap, decides membership by the exact test above and accumulates; a warp pays for it as
+// often as its busiest lane has survivors.
+//
+// What bounds it (720p, +-15, k = 7, FP32; ncu): instruction issue, 0.70 of the slots, with the filter
+// loop two thirds of the instructions (15 of 32 lanes active in it) and the loads' latency behind
+// the rest; DRAM at 8 %.  Testing the depth first, the short projection and x/y-paired filter
+// arithmetic took one 1080p +-30 frame from 5.47 to 3.97 ms, one 720p +-15 frame from 1.23 to 0.94 ms
+// (k = 5: 0.81 to 0.61), and the mixed clips' plan, 640 x 360 to 720p with FP16 colour, from 14.1 to 13.2.
 #include <cuda.h>  // CUtensorMap (the type only; the host encodes maps through the runtime's driver entry point)
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "../../include/ssvp.h"
 #include "ssvp_df.cuh"
@@ -31,14 +43,11 @@ namespace {
 #ifndef SSVP_MIN_CTAS
 #define SSVP_MIN_CTAS 4  // resident CTAs per SM the register allocation must allow
 #endif
-// The extraction gather of the learned filter keeps four more values live than the plain one; at
-// 64 registers (four CTAs per SM) it spills 80 bytes a thread, at 80 (three CTAs) 8.  Short windows,
-// whose accepted samples are nearly all stored, run faster with three CTAs and no spill traffic;
-// long ones, where the candidate loads dominate, with four CTAs and more warps to hide them.
-constexpr int kLearnCtasShort = 3;
-constexpr int kLearnShortSlots = 17;  // windows of up to +-8 frames
-
-
+// The extraction gather of the learned filter keeps more values live than the plain one: at 64 registers
+// (four CTAs per SM) it spills 96 bytes a thread, at 80 (three CTAs) none.  The gradient of a 16,384-pixel
+// batch of a 640 x 360 frame, +-15: 0.665 against 0.574 ms; a learned 1080p frame at +-30: 7.83 against
+// 7.77 ms, at +-6 3.96 against 3.96 ms.
+constexpr int kLearnCtas = 3;
 
 #ifndef SSVP_TILE_Y
 #define SSVP_TILE_Y 8  // output rows per CTA (a warp covers 32 pixels of one row)
@@ -106,9 +115,9 @@ __device__ __forceinline__ void stage_issue(const CUtensorMap *tmap, const float
     int x0 = kNoBox, y0 = kNoBox;
     if (J >= 0) {
         const float4 q0 = g[0], q1 = g[1], q2 = g[2], q3 = g[3];
-        const float w0 = fmaf(dref, q0.x + fmaf(q1.z, du, q1.w * dv), q3.x);
-        const float w1 = fmaf(dref, q0.y + fmaf(q2.x, du, q2.y * dv), q3.y);
-        const float w2 = fmaf(dref, q0.z + fmaf(q2.z, du, q2.w * dv), q3.z);
+        const float w0 = fmaf(dref, q0.x + fmaf(q1.x, du, q1.z * dv), q2.x);
+        const float w1 = fmaf(dref, q0.y + fmaf(q1.y, du, q1.w * dv), q2.y);
+        const float w2 = fmaf(dref, q3.x + fmaf(q3.z, du, q3.w * dv), g[4].x);
         if (w2 > 1e-6f * dref) {
             const float rz = rcp_approx(w2), U = w0 * rz, V = w1 * rz;
             if (fabsf(U) < 1e6f && fabsf(V) < 1e6f) {
@@ -168,19 +177,190 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     return y;
 }
 
+// How the test loop's survivors of a K x K window are kept: one bit per element of K rows of kC = K + 1
+// columns (aligned pairs of columns cover the window and one column beside it), in window order from
+// the top of the first word; kRows rows a word (7 x 8 bits need two words).
+template <int K>
+struct WindowBits {
+    static constexpr int kC = K + 1, kRows = K == 7 ? 4 : K, kWords = K == 7 ? 2 : 1;
+    static constexpr int kFill0 = 32 - kRows * kC, kFill1 = kWords == 2 ? 32 - (K - kRows) * kC : 0;
+    static constexpr unsigned rows_mask(int n) {
+        unsigned m = 0u;
+        for (int r = 0; r < n; ++r)
+            for (int c = 0; c < K; ++c) m |= 0x80000000u >> (r * kC + c);
+        return m;
+    }
+    static constexpr unsigned kMask0 = rows_mask(kRows), kMask1 = kWords == 2 ? rows_mask(K - kRows) : 0u;
+    // A bit's column and row, as exact floats and as the element offset row * pitch + col, from its index
+    // im (with the exponent bits of 2^23 set, its float form).  The row comes times kRowUnit: where a row
+    // has a power of two of bits, that is the index without its column bits.
+    static constexpr float kRowUnit = K == 5 ? 1.0f : (float)kC;
+    __device__ static __forceinline__ unsigned row5(unsigned im) { return ((im & 31u) * 43u) >> 8; }  // i / 6 for i < 32
+    __device__ static __forceinline__ unsigned col(unsigned im) {
+        return K == 5 ? im - 6u * row5(im) : (im & (kC - 1)) | kMagic;  // with the exponent bits too
+    }
+    __device__ static __forceinline__ f32x2 col_row(unsigned im) {
+        const float fc = __uint_as_float(col(im));
+        return f2_pack(fc - 8388608.0f, K == 5 ? small_float((int)row5(im)) : __uint_as_float(im) - fc);
+    }
+    __device__ static __forceinline__ unsigned offset(unsigned im, unsigned pitch) {
+        if (K == 5) return row5(im) * pitch + (col(im) - kMagic);
+        // index * (pitch / kC) + col * (1 - pitch / kC): the exponent bits enter once
+        return im * (pitch / kC) + (col(im) * (1u - pitch / kC) - kMagic);
+    }
+};
+template <>
+struct WindowBits<0> {};
+constexpr float kLateral = 4.0f;  // see lateral in gather_pixel
+
+// x_ref of the pixel (u0 + du, v0 + dv) at depth dref in the frame of slot geometry g: Z its depth
+// there and (U, V) its pixel position, as normalised double-float numbers; false when it lies behind
+// (or at) the camera.  m = M (u, v, 1) = M (u0, v0, 1) + M (du, dv, 0): the base in double-float, the
+// small offset exactly enough in FP32; w = dref m + e; U = w0 / w2, V = w1 / w2.  Only error-free
+// transformations and one correction step of the quotient; intermediate pairs are left unnormalised
+// (each low part is below 2^-22 of its high part), and x and y share packed operations.
+__device__ __forceinline__ bool project_slot(const float4 *g, const float4 q4, float du, float dv, float dref, df &Z, df &U,
+                                             df &V) {
+    const float4 q3 = g[3];
+    {
+        const df m = two_sum(q3.x, __fmaf_rn(q3.z, du, __fmul_rn(q3.w, dv)));
+        const df p = two_prod(m.hi, dref);
+        const float pl = __fmaf_rn(__fadd_rn(m.lo, q3.y), dref, p.lo);
+        const df s = two_sum(p.hi, q4.x);
+        Z = fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(pl, q4.y)));
+    }
+    if (!(Z.hi > 1e-6f * dref)) return false;
+    const float4 q0 = g[0], q1 = g[1], q2 = g[2];
+    const f32x2 mh = f2_pack(q0.x, q0.y), ml = f2_pack(q0.z, q0.w), eh = f2_pack(q2.x, q2.y), el = f2_pack(q2.z, q2.w);
+    const f32x2 t = f2_fma(f2_pack(q1.x, q1.y), f2_pack(du, du), f2_mul(f2_pack(q1.z, q1.w), f2_pack(dv, dv)));
+    // m = mh + t (two-sum) + ml
+    const f32x2 m = f2_add(mh, t), mb = f2_sub(m, mh);
+    const f32x2 me = f2_add(f2_add(f2_sub(mh, f2_sub(m, mb)), f2_sub(t, mb)), ml);
+    // w = m dref + e: -p is the rounded product's negative, so that the sum is a two-difference
+    const f32x2 d2 = f2_pack(dref, dref), np = f2_mul(m, f2_pack(-dref, -dref));
+    const f32x2 pl = f2_fma(me, d2, f2_fma(m, d2, np));
+    const f32x2 w = f2_sub(eh, np), wb = f2_sub(w, eh);  // wb: what of -np went into w
+    const f32x2 wl = f2_add(f2_sub(f2_sub(eh, f2_sub(w, wb)), f2_add(np, wb)), f2_add(pl, el));
+    // q = w / Z: first quotient -nq, remainder, correction
+    const float r = rcp_approx(Z.hi);
+    const f32x2 zh2 = f2_pack(Z.hi, Z.hi), nq = f2_mul(w, f2_pack(-r, -r));
+    const f32x2 rem = f2_fma(nq, f2_pack(Z.lo, Z.lo), f2_add(f2_fma(nq, zh2, w), wl));
+    const f32x2 c = f2_mul(rem, f2_pack(r, r));
+    const f32x2 hi = f2_sub(c, nq), lo = f2_sub(c, f2_add(hi, nq));
+    f2_unpack(hi, U.hi, V.hi);
+    f2_unpack(lo, U.lo, V.lo);
+    return true;
+}
+
+// The test loops of a K x K window whose even-column rows start at dtest (pitch tpitch): one bit per
+// element of K rows of K + 1 columns, the sign of the tested quantity shifted in, window order from
+// the top of the words (not yet top-aligned, the spare column not yet masked).
+// By depth: e^2 - thr, e = d - zh; nthr = -thr.
+template <int K, bool STG>
+__device__ __forceinline__ void test_depth(const float *dtest, long long tpitch, float zh, float nthr, unsigned (&m)[2]) {
+    const f32x2 zh2 = f2_pack(zh, zh), nthr2 = f2_pack(nthr, nthr);
+    m[0] = m[1] = 0u;
+#pragma unroll
+    for (int dy = 0; dy < K; ++dy) {
+        const f32x2 *drow = reinterpret_cast<const f32x2 *>(dtest + (long long)dy * tpitch);
+        unsigned &mw = m[dy / WindowBits<K>::kRows];
+#pragma unroll
+        for (int q = 0; q < (K + 1) / 2; ++q) {
+            // staged: a generic load (shared memory, or the global plane outside the box)
+            const f32x2 e = f2_sub(STG ? drow[q] : __ldg(drow + q), zh2);
+            float ta, tb;
+            f2_unpack(f2_fma(e, e, nthr2), ta, tb);
+            mw = __funnelshift_l(__float_as_uint(ta), mw, 1);
+            mw = __funnelshift_l(__float_as_uint(tb), mw, 1);
+        }
+    }
+}
+
+// By the whole distance: e^2 + X^2 + Y^2 - r^2 with (ax, ifx), (bx, zix), (ay, ify), (by, ziy) giving X
+// and Y as in the exact test, ax and bx at the even column; lim bounds |By| of the rows that can hold a
+// sample.  ROWS rows at a time, those that no lane of the warp needs left out: all seven at once take
+// more registers than the kernel has (112 bytes spilled), and so do two with the three records in flight
+// of the FP32 filter loop (1080p +-30: 3.97 against 4.11 ms).  Two where they fit hide more of the loads'
+// latency: the mixed clips' plan 13.2 against 13.9 ms.
+template <int K, int ROWS, bool STG>
+__device__ __forceinline__ void test_distance(const float *dtest, long long tpitch, float zh, float r, float lim, float ax,
+                                              float ifx, float bx, float zix, float ay, float ify, float by, float ziy,
+                                              unsigned (&m)[2]) {
+    using WB = WindowBits<K>;
+    constexpr int KP = (K + 1) / 2;
+    const float nthr = -(r * r);
+    const f32x2 zh2 = f2_pack(zh, zh), nthr2 = f2_pack(nthr, nthr);
+    f32x2 Ax[KP], Bx[KP];
+#pragma unroll
+    for (int q = 0; q < KP; ++q) {
+        Ax[q] = f2_pack(__fmaf_rn((float)(2 * q), ifx, ax), __fmaf_rn((float)(2 * q + 1), ifx, ax));
+        Bx[q] = f2_pack(__fmaf_rn((float)(2 * q), zix, bx), __fmaf_rn((float)(2 * q + 1), zix, bx));
+    }
+    auto rows = [&](int dy, auto n_rows, unsigned &mw) {
+        constexpr int N = decltype(n_rows)::value;
+        const float By0 = __fmaf_rn((float)dy, ziy, by), By1 = __fmaf_rn((float)(dy + N - 1), ziy, by);
+        if (!__any_sync(__activemask(), By0 <= lim && By1 >= -lim)) {
+            mw <<= N * WB::kC;
+            return;
+        }
+        f32x2 e[N][KP];
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int q = 0; q < KP; ++q) {
+                const f32x2 *p = reinterpret_cast<const f32x2 *>(dtest + (long long)(dy + i) * tpitch) + q;
+                e[i][q] = f2_sub(STG ? *p : __ldg(p), zh2);
+            }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float Ay = __fmaf_rn((float)(dy + i), ify, ay), By = i == 0 ? By0 : By1;
+#pragma unroll
+            for (int q = 0; q < KP; ++q) {
+                const f32x2 X = f2_fma(e[i][q], Ax[q], Bx[q]), Y = f2_fma(e[i][q], f2_pack(Ay, Ay), f2_pack(By, By));
+                float ta, tb;
+                f2_unpack(f2_fma(X, X, f2_fma(Y, Y, f2_fma(e[i][q], e[i][q], nthr2))), ta, tb);
+                mw = __funnelshift_l(__float_as_uint(ta), mw, 1);
+                mw = __funnelshift_l(__float_as_uint(tb), mw, 1);
+            }
+        }
+    };
+    using One = std::integral_constant<int, 1>;
+    using Two = std::integral_constant<int, 2>;
+    m[0] = m[1] = 0u;
+    if (ROWS == 1) {
+#pragma unroll 1
+        for (int dy = 0; dy < WB::kRows; ++dy) rows(dy, One{}, m[0]);
+#pragma unroll 1
+        for (int dy = WB::kRows; dy < K; ++dy) rows(dy, One{}, m[1]);
+    } else {
+#pragma unroll 1
+        for (int dy = 0; dy + 1 < WB::kRows; dy += 2) rows(dy, Two{}, m[0]);
+        if (WB::kRows & 1) rows(WB::kRows - 1, One{}, m[0]);
+        if (K == 7) {
+            rows(4, Two{}, m[1]);
+            rows(6, One{}, m[1]);
+        }
+    }
+}
+
 // LEARN: visit the frames in canonical order (O, O-1, O+1, ...) and store the features of the
 // first kMaxSamples accepted samples (learned filter); the Eq. 3/4 result goes to a.sets.plain.
-// ACCB: accepted samples taken per iteration of the filter loop of a compile-time window (1, or
-// 2 in packed FP32x2, which the kernels use; the runtime-k path takes them one at a time)
 // STG: the candidate depths of the test loop come from the warp's staged boxes (K > 0, not LEARN);
 // tmap describes the clip's depth planes
-template <int K, int CFMT, bool DEBUG, bool LEARN = false, int ACCB = 1, bool STG = false>
+// a_rgb and a_xyz: -log2(e) / (2 sigma^2) of Eq. 4's colour and position terms
+// NS: survivors per iteration of the filter loop of a compile-time window.  Each is one more record in
+// flight and up to NS - 1 idle slots at the end of a frame's list: 2 -> 3 takes a 1080p +-30 FP32 frame
+// from 4.15 to 3.99 ms, but with FP16 colour, whose samples take two loads and conversions, and in the
+// batched kernel the registers run out (a 720p FP16 frame 1.03 -> 1.06 ms, the mixed clips' plan 13.5 -> 14.0)
+template <int K, int CFMT, int NS, bool DEBUG, bool LEARN = false, bool STG = false>
 __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &P, const int O, const int u0,
                                              const int v0, const int u, const int v, const bool active,
                                              const long long crop_idx, const float4 *sgeom, const int n_slots,
                                              const float r2, const float a_rgb, const float a_xyz, const bool weighted,
-                                             int &n_acc, int &n_exam, float &acc_w, const CUtensorMap *tmap = nullptr) {
+                                             float &n_acc, int &n_exam, float &acc_w, const CUtensorMap *tmap = nullptr) {
     static_assert(!STG || (K > 0 && K <= kStageMaxK && !LEARN), "staging: compile-time k <= 7, plain gather");
+    using WB = WindowBits<K>;
+    constexpr int kTestRows = K == 7 && (NS == 2 || LEARN) ? 2 : 1;  // see test_distance
     const int k = K > 0 ? K : a.k;
     const int h = (k - 1) >> 1;
     const int rec_words = 3 + (k * k + 31) / 32;
@@ -197,6 +377,19 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
         cref = load_colour<CFMT>(P.colour, pix);
     }
     const bool gather = active && dref > 0.0f;  // false for NaN (invalid) depth
+    const float r_up = __fsqrt_rn(r2) * 1.000001f;
+    // Which test the warp's windows get.  Depth alone costs 2 packed operations per pair of columns and
+    // lets through candidates inside the depth slab but off to the side; the whole distance costs 6.
+    // The first is better unless the window's corners lie well outside the radius: at (corner distance)^2
+    // = 4 r^2 (r = 2.5 pixels with k = 7) the two tie (640 x 360 +-15, 8 frames: 1.83 ms with the line at
+    // 3, 4 or 6); 160 x 90 with k = 5 (r = 0.6 pixels) takes 0.100 with the whole distance and 0.152 ms by
+    // depth, 1080p (r = 7 pixels) 5.03 and 4.16 ms.
+    bool lateral = false;
+    {
+        const float4 qc = sgeom[kSlotVec * ((n_slots - 1) >> 1) + 4];
+        const float bx = (0.5f * (float)k) * dref * qc.z, by = (0.5f * (float)k) * dref * qc.w;
+        lateral = __any_sync(0xffffffffu, gather && fmaf(bx, bx, by * by) > kLateral * r2);
+    }
     // staging: the warp's gathering lanes, the first of them issues the copies
     const unsigned G = STG ? __ballot_sync(0xffffffffu, gather) : 0u;
     int stg_fail = -1;  // staging: the slot whose wait gave up (-1: staging on)
@@ -235,258 +428,230 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
                 if (DEBUG && rec) rec[0] = -1;
                 continue;
             }
-            const float4 q0 = g[0], q1 = g[1], q2 = g[2], q3 = g[3], q4 = g[4];
-            // m = M (u, v, 1) = M (u0, v0, 1) + M (du, dv, 0): the base in double-float, the small
-            // offset exactly enough in FP32
-            df m0 = df_add_f({q0.x, q0.w}, __fmaf_rn(q1.z, du, __fmul_rn(q1.w, dv)));
-            df m1 = df_add_f({q0.y, q1.x}, __fmaf_rn(q2.x, du, __fmul_rn(q2.y, dv)));
-            df m2 = df_add_f({q0.z, q1.y}, __fmaf_rn(q2.z, du, __fmul_rn(q2.w, dv)));
-            // w = d_ref m + e: homogeneous pixel coordinates of x_ref in J
-            df w0 = df_add(df_mul_f(m0, dref), {q3.x, q3.w});
-            df w1 = df_add(df_mul_f(m1, dref), {q3.y, q4.x});
-            df w2 = df_add(df_mul_f(m2, dref), {q3.z, q4.y});
-            if (!(w2.hi > 1e-6f * dref)) {  // behind (or at) camera J
+            const float4 q4 = g[4];
+            df Z, U, V;
+            if (!project_slot(g, q4, du, dv, dref, Z, U, V)) {  // behind (or at) camera J
                 if (DEBUG && rec) rec[0] = 0;
                 continue;
             }
-            const float rz = rcp_approx(w2.hi);
-            const df U = df_div(w0, w2, rz), V = df_div(w1, w2, rz);
             // window centre floor(u' + 0.5) and the exact offset u' - centre in [-0.5, 0.5)
             float cxf = floorf(U.hi + 0.5f), cyf = floorf(V.hi + 0.5f);
             float ou = __fadd_rn(__fsub_rn(U.hi, cxf), U.lo), ov = __fadd_rn(__fsub_rn(V.hi, cyf), V.lo);
-            if (ou < -0.5f) { cxf -= 1.0f; ou += 1.0f; } else if (ou >= 0.5f) { cxf += 1.0f; ou -= 1.0f; }
-            if (ov < -0.5f) { cyf -= 1.0f; ov += 1.0f; } else if (ov >= 0.5f) { cyf += 1.0f; ov -= 1.0f; }
+            if (!(fabsf(ou) < 0.5f && fabsf(ov) < 0.5f)) {
+                if (ou < -0.5f) { cxf -= 1.0f; ou += 1.0f; } else if (ou >= 0.5f) { cxf += 1.0f; ou -= 1.0f; }
+                if (ov < -0.5f) { cyf -= 1.0f; ov += 1.0f; } else if (ov >= 0.5f) { cyf += 1.0f; ov -= 1.0f; }
+            }
             if (!(cxf >= (float)-h && cxf <= (float)(P.W - 1 + h) && cyf >= (float)-h && cyf <= (float)(P.H - 1 + h))) {
                 if (DEBUG && rec) { rec[0] = 2; }
                 continue;  // no window pixel inside the image
             }
             const int cx = (int)cxf, cy = (int)cyf;
-            {
+            if ((unsigned)(cx - h) < (unsigned)max(P.W - k + 1, 0) && (unsigned)(cy - h) < (unsigned)max(P.H - k + 1, 0)) {
+                n_exam += k * k;
+            } else {
                 int nx = min(cx + h, P.W - 1) - max(cx - h, 0) + 1;
                 int ny = min(cy + h, P.H - 1) - max(cy - h, 0) + 1;
                 n_exam += nx * ny;
             }
             const float ifx = q4.z, ify = q4.w;
-            const float zh = w2.hi, zl = w2.lo;
+            const float zh = Z.hi, zl = Z.lo;
             // ray_x(q) = (q_x - cx_J) / fx and z' (q_x - u') / fx as affine functions of dx
             const float Ax0 = (cxf - (float)h - q5.x) * ifx, zix = zh * ifx, Bx0 = (-(float)h - ou) * zix;
             const float Ay0 = (cyf - (float)h - q5.y) * ify, ziy = zh * ify, By0 = (-(float)h - ov) * ziy;
-            const long long wbase = (long long)J * P.fstride + (long long)(cy - h + kPad) * P.pitch + (cx - h + kPad);
-            const float *dwin = P.depth + wbase;
-            const void *cwin = CFMT == 0 ? (const void *)(reinterpret_cast<const float4 *>(P.colour) + wbase)
-                                         : (const void *)(reinterpret_cast<const uint2 *>(P.colour) + wbase);
-            const float beta = q5.z;
+            // the window's first element, and the even column at or before it (xw - par): the test
+            // loop's loads are aligned pairs of columns
+            const int xw = cx - h + kPad, yw = cy - h + kPad, par = xw & 1;
+            const long long fbase = (long long)J * P.fstride;
+            const int woff = yw * P.pitch + xw;
+            const float *dwin = P.depth + fbase + woff;
+            const void *cwin = CFMT == 0 ? (const void *)(reinterpret_cast<const float4 *>(P.colour) + fbase + woff)
+                                         : (const void *)(reinterpret_cast<const uint2 *>(P.colour) + fbase + woff);
+            const float beta = -q5.z;
             const float dj_t = LEARN ? (float)(j - Tw) * inv_T : 0.0f;  // the frame-offset feature
-            if (DEBUG && rec) { rec[0] = 1; rec[1] = cx; rec[2] = cy; }
-
-            if (K > 0) {
+            if (DEBUG && rec) {
+                rec[0] = 1; rec[1] = cx; rec[2] = cy;
+                for (int wd = 3; wd < rec_words; ++wd) rec[wd] = 0;
+            }
+            // The depth test |d_q - z'| < r is necessary for the radius test (d^2 >= dz^2 in FP32 too: the
+            // other terms are added to it).  It is evaluated as e^2 < thr, e = d_q - zh without the low
+            // part of z': thr = (r + |zl|)^2 with its roundings covered.
+            const float rc = fmaf(fabsf(zl), 1.000001f, r_up), nthr = -(rc * rc) * 1.000001f;
+            // the whole distance with e for dz: the difference, |zl| times the slopes of X and Y, and the
+            // roundings, which grow with the slopes, widen the radius; |Y| < r bounds |By| by r + |e Ay|
+            const float sl = 1.0f + fabsf(Ax0) + fabsf(Ay0) + (float)k * (ifx + ify);
+            const float rl = fmaf(fabsf(zl), sl, r_up) * fmaf(sl, 2e-6f, 1.0f), lim = rl * (sl - fabsf(Ax0)) * 1.0001f;
+            if constexpr (K > 0) {
                 // the test loop's depths: this lane's window in the staged box if it lies inside it
-                const float *dtest = dwin;
+                const float *dtest = dwin - par;
                 long long tpitch = P.pitch;
                 if (STG) {
-                    const int ox = cx - h + kPad - org.x, oy = cy - h + kPad - org.y;
+                    const int ox = xw - org.x, oy = yw - org.y;
                     if ((unsigned)ox <= (unsigned)(kBoxW - K) && (unsigned)oy <= (unsigned)(kBoxH - K)) {
+                        // box columns start at a multiple of four, so ox has the parity of xw
                         dtest = reinterpret_cast<const float *>(reinterpret_cast<const char *>(sgeom) +
                                                                 (stg_box(sgeom, n_slots, jj & 1) - smem_addr(sgeom))) +
-                                oy * kBoxW + ox;
+                                oy * kBoxW + (ox - par);
                         tpitch = kBoxW;
                     }
                 }
-                float Ax[K > 0 ? K : 1], Bx[K > 0 ? K : 1];
+                unsigned m[2];
+                if (lateral)
+                    test_distance<K, kTestRows, STG>(dtest, tpitch, zh, rl, lim, fmaf(-(float)par, ifx, Ax0), ifx,
+                                          fmaf(-(float)par, zix, Bx0), zix, Ay0, ify, By0, ziy, m);
+                else
+                    test_depth<K, STG>(dtest, tpitch, zh, nthr, m);
+                // top-aligned, the spare column (the last one, or the first if the window starts at an odd
+                // element) out: bit i of the words, from the top, is window element (i / (K + 1), i % (K + 1))
+                m[0] = ((m[0] << WB::kFill0) << par) & WB::kMask0;
+                m[1] = ((m[1] << WB::kFill1) << par) & WB::kMask1;
+                unsigned acc_bits[2] = {0u, 0u};  // DEBUG: the accepted ones of m
+                // LEARN keeps the sums of a frame's even and odd accepted samples apart, folded after the
+                // frame, in whatever pairs the survivors come (the stored features and the plain result
+                // do not depend on how the test loop selects them)
+                float s_r[2] = {0.f, 0.f}, s_g[2] = {0.f, 0.f}, s_b[2] = {0.f, 0.f}, s_w[2] = {0.f, 0.f};
+                bool odd = false;
+                // The survivors, NS per iteration so that their loads overlap: the exact radius test, then
+                // the filter.  x and y of a sample share packed operations, and so do the halves of its
+                // 16-byte record, (r, g) and (b, depth), as they are loaded.
+                constexpr float kRowScale = 1.0f / WB::kRowUnit;
+                const f32x2 step_a = f2_pack(ifx, ify * kRowScale), step_b = f2_pack(zix, ziy * kRowScale);
+                const f32x2 a0 = f2_pack(Ax0, Ay0), b0 = f2_pack(Bx0, By0);
+                const f32x2 ref_rg = f2_pack(cref.x, cref.y), ref_bz = f2_pack(cref.z, zh);
+                int pos = 0;
+#pragma unroll 1
+                while (WB::kWords == 2 ? (m[0] | m[1]) != 0u : m[0] != 0u) {
+                    unsigned im[NS];
+                    bool ok[NS];
+                    f32x2 rg[NS], bz[NS];
 #pragma unroll
-                for (int dx = 0; dx < K; ++dx) {
-                    Ax[dx] = __fmaf_rn((float)dx, ifx, Ax0);
-                    Bx[dx] = __fmaf_rn((float)dx, zix, Bx0);
-                }
-                // columns (dx, dx + 1) are tested as pairs with packed FP32x2 arithmetic: each half
-                // runs the scalar sequence below, so the distances are the same to the bit
-                constexpr int KP = K / 2;
-                f32x2 AxP[KP > 0 ? KP : 1], BxP[KP > 0 ? KP : 1];
-#pragma unroll
-                for (int q = 0; q < KP; ++q) {
-                    AxP[q] = f2_pack(Ax[2 * q], Ax[2 * q + 1]);
-                    BxP[q] = f2_pack(Bx[2 * q], Bx[2 * q + 1]);
-                }
-                const f32x2 zh2 = f2_pack(zh, zh), zl2 = f2_pack(zl, zl);
-                unsigned long long mask = 0ull;
-#pragma unroll
-                for (int dy = 0; dy < K; ++dy) {
-                    const float Ay = __fmaf_rn((float)dy, ify, Ay0), By = __fmaf_rn((float)dy, ziy, By0);
-                    const f32x2 Ay2 = f2_pack(Ay, Ay), By2 = f2_pack(By, By);
-                    const float *drow = dtest + (long long)dy * tpitch;
-#pragma unroll
-                    for (int q = 0; q < KP; ++q) {
-                        // staged: a generic load (shared memory, or the global plane outside the box)
-                        const float da = STG ? drow[2 * q] : __ldg(drow + 2 * q);
-                        const float db = STG ? drow[2 * q + 1] : __ldg(drow + 2 * q + 1);
-                        const f32x2 dz = f2_sub(f2_sub(f2_pack(da, db), zh2), zl2);
-                        const f32x2 X = f2_fma(dz, AxP[q], BxP[q]);
-                        const f32x2 Y = f2_fma(dz, Ay2, By2);
-                        const f32x2 d2 = f2_fma(X, X, f2_fma(Y, Y, f2_mul(dz, dz)));
-                        float d2a, d2b;
-                        f2_unpack(d2, d2a, d2b);
-                        if (d2a < r2) mask |= 1ull << (dy * 8 + 2 * q);  // stride 8: cheap decode
-                        if (d2b < r2) mask |= 1ull << (dy * 8 + 2 * q + 1);
+                    for (int t = 0; t < NS; ++t) {
+                        // the next bit goes to the top; a step over 32 zeros finds none (ok false)
+                        const int c = __clz((int)m[0]);
+                        pos += c;
+                        const unsigned top = __funnelshift_lc(WB::kWords == 2 ? m[1] : 0u, m[0], c);
+                        if (WB::kWords == 2) m[1] = __funnelshift_lc(0u, m[1], c);
+                        m[0] = top & 0x7fffffffu;
+                        ok[t] = (int)top < 0;
+                        im[t] = ((unsigned)pos & (WB::kWords * 32 - 1)) | kMagic;  // any value stays inside the padded plane
+                        load_record<CFMT>(dwin, cwin, (int)WB::offset(im[t], P.pitch), rg[t], bz[t]);
                     }
-                    if (K & 1) {
-                        constexpr int dx = K - 1;
-                        const float dz = ((STG ? drow[dx] : __ldg(drow + dx)) - zh) - zl;
-                        const float X = fmaf(dz, Ax[dx], Bx[dx]);
-                        const float Y = fmaf(dz, Ay, By);
+#pragma unroll
+                    for (int t = 0; t < NS; ++t) {
+                        const f32x2 xy = WB::col_row(im[t]);
+                        const f32x2 erg = f2_sub(rg[t], ref_rg), ebz = f2_sub(bz[t], ref_bz);
+                        float er, eg, eb, dz, X, Y;
+                        f2_unpack(erg, er, eg);
+                        f2_unpack(ebz, eb, dz);
+                        dz = dz - zl;
+                        const f32x2 XY = f2_fma(f2_pack(dz, dz), f2_fma(xy, step_a, a0), f2_fma(xy, step_b, b0));
+                        f2_unpack(XY, X, Y);
                         const float d2 = fmaf(X, X, fmaf(Y, Y, dz * dz));
-                        if (d2 < r2) mask |= 1ull << (dy * 8 + dx);
+                        // log2 of the weight (a_rgb and a_xyz are negative, beta is minus the frame term)
+                        const float e = fmaf(a_rgb, fmaf(er, er, fmaf(eg, eg, eb * eb)), fmaf(a_xyz, d2, beta));
+                        const float w = weighted ? ex2(e) : 1.0f;
+                        if (ok[t] && d2 < r2) {
+                            n_acc += 1.0f;
+                            if (DEBUG) acc_bits[(im[t] >> 5) & 1] |= 0x80000000u >> (im[t] & 31);
+                            if (!LEARN) {
+                                acc_r = fmaf(w, er, acc_r);
+                                acc_g = fmaf(w, eg, acc_g);
+                                acc_b = fmaf(w, eb, acc_b);
+                                acc_w += w;
+                            } else {
+                                if (n_feat < kMaxSamples) {
+                                    float cr, cg, cb, cd;
+                                    f2_unpack(rg[t], cr, cg);
+                                    f2_unpack(bz[t], cb, cd);
+                                    store_sample(a, set0 + n_feat, make_float3(cr, cg, cb), sqrt_approx(d2) * inv_r, dj_t,
+                                                 dz * inv_r, e * kLn2);
+                                    ++n_feat;
+                                }
+                                s_r[0] = odd ? s_r[0] : fmaf(w, er, s_r[0]);
+                                s_r[1] = odd ? fmaf(w, er, s_r[1]) : s_r[1];
+                                s_g[0] = odd ? s_g[0] : fmaf(w, eg, s_g[0]);
+                                s_g[1] = odd ? fmaf(w, eg, s_g[1]) : s_g[1];
+                                s_b[0] = odd ? s_b[0] : fmaf(w, eb, s_b[0]);
+                                s_b[1] = odd ? fmaf(w, eb, s_b[1]) : s_b[1];
+                                s_w[0] += odd ? 0.0f : w;
+                                s_w[1] += odd ? w : 0.0f;
+                                odd = !odd;
+                            }
+                        }
                     }
+                }
+                if (LEARN) {
+                    acc_r += s_r[0] + s_r[1];
+                    acc_g += s_g[0] + s_g[1];
+                    acc_b += s_b[0] + s_b[1];
+                    acc_w += s_w[0] + s_w[1];
                 }
                 if (DEBUG && rec) {
-                    unsigned long long packed = 0ull;  // record layout: bit dy*k+dx
-                    for (int dy = 0; dy < K; ++dy)
-                        packed |= ((mask >> (8 * dy)) & ((1ull << K) - 1ull)) << (dy * K);
-                    rec[3] = (int32_t)(unsigned int)(packed & 0xffffffffull);
-                    if (K * K > 32) rec[4] = (int32_t)(unsigned int)(packed >> 32);
-                }
-                // accepted samples, ACCB per iteration so that their loads overlap; with two,
-                // the pair's sums are kept in packed partial sums and folded after the frame
-                f32x2 pr = 0ull, pg = 0ull, pb = 0ull, pw = 0ull;  // +0.0f in both halves
-#pragma unroll 1
-                while (mask) {
-                    int idx[ACCB];
-                    bool ok[ACCB];
-#pragma unroll
-                    for (int t = 0; t < ACCB; ++t) {
-                        ok[t] = mask != 0ull;
-                        idx[t] = ok[t] ? __ffsll((long long)mask) - 1 : 0;  // slot 0 is always in bounds
-                        mask &= mask - 1ull;
-                    }
-                    float dq[ACCB];
-                    float3 cq[ACCB];
-#pragma unroll
-                    for (int t = 0; t < ACCB; ++t) {
-                        const int off = (idx[t] >> 3) * P.pitch + (idx[t] & 7);
-                        load_sample<CFMT>(dwin, cwin, off, dq[t], cq[t]);
-                    }
-                    if constexpr (ACCB == 2) {
-                        // the two samples in packed FP32x2: per half the scalar sequence below
-                        const f32x2 dxf = f2_pack(small_float(idx[0] & 7), small_float(idx[1] & 7));
-                        const f32x2 dyf = f2_pack(small_float(idx[0] >> 3), small_float(idx[1] >> 3));
-                        const f32x2 dz = f2_sub(f2_sub(f2_pack(dq[0], dq[1]), f2_pack(zh, zh)), f2_pack(zl, zl));
-                        const f32x2 X = f2_fma(dz, f2_fma(dxf, f2_pack(ifx, ifx), f2_pack(Ax0, Ax0)),
-                                               f2_fma(dxf, f2_pack(zix, zix), f2_pack(Bx0, Bx0)));
-                        const f32x2 Y = f2_fma(dz, f2_fma(dyf, f2_pack(ify, ify), f2_pack(Ay0, Ay0)),
-                                               f2_fma(dyf, f2_pack(ziy, ziy), f2_pack(By0, By0)));
-                        const f32x2 d2 = f2_fma(X, X, f2_fma(Y, Y, f2_mul(dz, dz)));
-                        const f32x2 er = f2_sub(f2_pack(cq[0].x, cq[1].x), f2_pack(cref.x, cref.x));
-                        const f32x2 eg = f2_sub(f2_pack(cq[0].y, cq[1].y), f2_pack(cref.y, cref.y));
-                        const f32x2 eb = f2_sub(f2_pack(cq[0].z, cq[1].z), f2_pack(cref.z, cref.z));
-                        const f32x2 e = f2_fma(f2_pack(a_rgb, a_rgb), f2_fma(er, er, f2_fma(eg, eg, f2_mul(eb, eb))),
-                                               f2_fma(f2_pack(a_xyz, a_xyz), d2, f2_pack(beta, beta)));
-                        float e0, e1;
-                        f2_unpack(e, e0, e1);
-                        const float w0 = weighted ? ex2(-e0) : 1.0f;
-                        const float w1 = ok[1] ? (weighted ? ex2(-e1) : 1.0f) : 0.0f;  // ok[0] holds in the loop
-                        if (LEARN) {
-                            float dd0, dd1, dz0, dz1;
-                            f2_unpack(d2, dd0, dd1);
-                            f2_unpack(dz, dz0, dz1);
-                            if (n_feat < kMaxSamples) {
-                                store_sample(a, set0 + n_feat, cq[0], sqrt_approx(dd0) * inv_r, dj_t, dz0 * inv_r,
-                                             -e0 * kLn2);
-                                ++n_feat;
-                            }
-                            if (ok[1] && n_feat < kMaxSamples) {
-                                store_sample(a, set0 + n_feat, cq[1], sqrt_approx(dd1) * inv_r, dj_t, dz1 * inv_r,
-                                             -e1 * kLn2);
-                                ++n_feat;
-                            }
+                    for (int i = 0; i < K * WB::kC; ++i)  // record layout: bit dy*k+dx
+                        if (acc_bits[i >> 5] << (i & 31) >> 31) {
+                            const int bit = i / WB::kC * K + i % WB::kC;
+                            rec[3 + (bit >> 5)] |= (int32_t)(1u << (bit & 31));
                         }
-                        const f32x2 w = f2_pack(w0, w1);
-                        pr = f2_fma(w, er, pr);
-                        pg = f2_fma(w, eg, pg);
-                        pb = f2_fma(w, eb, pb);
-                        pw = f2_add(pw, w);
-                        n_acc += 1 + (ok[1] ? 1 : 0);
-                    } else {
-#pragma unroll
-                    for (int t = 0; t < ACCB; ++t) {
-                        const float dxf = small_float(idx[t] & 7), dyf = small_float(idx[t] >> 3);
-                        const float dz = (dq[t] - zh) - zl;
-                        const float X = fmaf(dz, __fmaf_rn(dxf, ifx, Ax0), __fmaf_rn(dxf, zix, Bx0));
-                        const float Y = fmaf(dz, __fmaf_rn(dyf, ify, Ay0), __fmaf_rn(dyf, ziy, By0));
-                        const float d2 = fmaf(X, X, fmaf(Y, Y, dz * dz));
-                        const float er = cq[t].x - cref.x, eg = cq[t].y - cref.y, eb = cq[t].z - cref.z;
-                        const float e = fmaf(a_rgb, fmaf(er, er, fmaf(eg, eg, eb * eb)), fmaf(a_xyz, d2, beta));
-                        float w = 1.0f;
-                        if (weighted) w = ex2(-e);
-                        if (LEARN && ok[t] && n_feat < kMaxSamples) {
-                            store_sample(a, set0 + n_feat, cq[t], sqrt_approx(d2) * inv_r, dj_t, dz * inv_r,
-                                         -e * kLn2);
-                            ++n_feat;
-                        }
-                        if (ok[t]) {
-                            acc_r = fmaf(w, er, acc_r);
-                            acc_g = fmaf(w, eg, acc_g);
-                            acc_b = fmaf(w, eb, acc_b);
-                            acc_w += w;
-                            ++n_acc;
-                        }
-                    }
-                    }
-                }
-                if (ACCB == 2) {
-                    float lo, hi;
-                    f2_unpack(pr, lo, hi);
-                    acc_r += lo + hi;
-                    f2_unpack(pg, lo, hi);
-                    acc_g += lo + hi;
-                    f2_unpack(pb, lo, hi);
-                    acc_b += lo + hi;
-                    f2_unpack(pw, lo, hi);
-                    acc_w += lo + hi;
                 }
             } else {
-                if (DEBUG && rec)
-                    for (int wd = 3; wd < rec_words; ++wd) rec[wd] = 0;
                 for (int dy = 0; dy < k; ++dy) {
                     const float Ay = __fmaf_rn((float)dy, ify, Ay0), By = __fmaf_rn((float)dy, ziy, By0);
-                    const float *drow = dwin + (long long)dy * P.pitch;
+                    // k + 1 columns (at most 32) from the even one, one bit each, top-aligned
+                    const f32x2 *drow = reinterpret_cast<const f32x2 *>(dwin - par + (long long)dy * P.pitch);
+                    const f32x2 zh2 = f2_pack(zh, zh);
                     unsigned int mask = 0u;
-                    for (int dx = 0; dx < k; ++dx) {
-                        const float dz = (__ldg(drow + dx) - zh) - zl;
-                        const float X = fmaf(dz, __fmaf_rn((float)dx, ifx, Ax0), __fmaf_rn((float)dx, zix, Bx0));
-                        const float Y = fmaf(dz, Ay, By);
-                        const float d2 = fmaf(X, X, fmaf(Y, Y, dz * dz));
-                        if (d2 < r2) mask |= 1u << dx;
+                    if (lateral) {
+                        if (!__any_sync(__activemask(), fabsf(By) <= lim)) continue;
+                        const f32x2 nthr2 = f2_pack(-(rl * rl), -(rl * rl)), Ay2 = f2_pack(Ay, Ay), By2 = f2_pack(By, By);
+                        const float axe = fmaf(-(float)par, ifx, Ax0), bxe = fmaf(-(float)par, zix, Bx0);
+                        for (int q = 0; q < (k + 1) >> 1; ++q) {
+                            const f32x2 e = f2_sub(__ldg(drow + q), zh2), c = f2_pack((float)(2 * q), (float)(2 * q + 1));
+                            const f32x2 X = f2_fma(e, f2_fma(c, f2_pack(ifx, ifx), f2_pack(axe, axe)),
+                                                   f2_fma(c, f2_pack(zix, zix), f2_pack(bxe, bxe)));
+                            const f32x2 Y = f2_fma(e, Ay2, By2);
+                            float ta, tb;
+                            f2_unpack(f2_fma(X, X, f2_fma(Y, Y, f2_fma(e, e, nthr2))), ta, tb);
+                            mask = __funnelshift_l(__float_as_uint(ta), mask, 1);
+                            mask = __funnelshift_l(__float_as_uint(tb), mask, 1);
+                        }
+                    } else {
+                        const f32x2 nthr2 = f2_pack(nthr, nthr);
+                        for (int q = 0; q < (k + 1) >> 1; ++q) {
+                            const f32x2 e = f2_sub(__ldg(drow + q), zh2);
+                            float ta, tb;
+                            f2_unpack(f2_fma(e, e, nthr2), ta, tb);
+                            mask = __funnelshift_l(__float_as_uint(ta), mask, 1);
+                            mask = __funnelshift_l(__float_as_uint(tb), mask, 1);
+                        }
                     }
-                    if (DEBUG && rec) {
-                        for (int dx = 0; dx < k; ++dx)
-                            if (mask >> dx & 1u) {
-                                const int bit = dy * k + dx;
-                                rec[3 + (bit >> 5)] |= (int32_t)(1u << (bit & 31));
-                            }
-                    }
+                    mask = ((mask << (31 - k)) << par) & (0xffffffffu << (32 - k));
                     while (mask) {
-                        const int dx = __ffs((int)mask) - 1;
-                        mask &= mask - 1u;
-                        const long long off = (long long)dy * P.pitch + dx;
+                        const int dx = __clz((int)mask);
+                        mask &= 0x7fffffffu >> dx;
                         float dq;
                         float3 c;
-                        load_sample<CFMT>(dwin, cwin, off, dq, c);
+                        load_sample<CFMT>(dwin, cwin, dy * P.pitch + dx, dq, c);
                         const float dz = (dq - zh) - zl;
                         const float X = fmaf(dz, __fmaf_rn((float)dx, ifx, Ax0), __fmaf_rn((float)dx, zix, Bx0));
                         const float Y = fmaf(dz, Ay, By);
                         const float d2 = fmaf(X, X, fmaf(Y, Y, dz * dz));
+                        if (!(d2 < r2)) continue;
+                        if (DEBUG && rec) {
+                            const int bit = dy * k + dx;
+                            rec[3 + (bit >> 5)] |= (int32_t)(1u << (bit & 31));
+                        }
                         const float er = c.x - cref.x, eg = c.y - cref.y, eb = c.z - cref.z;
                         const float e = fmaf(a_rgb, fmaf(er, er, fmaf(eg, eg, eb * eb)), fmaf(a_xyz, d2, beta));
                         float w = 1.0f;
-                        if (weighted) w = ex2(-e);
+                        if (weighted) w = ex2(e);
                         if (LEARN && n_feat < kMaxSamples) {
-                            store_sample(a, set0 + n_feat, c, sqrt_approx(d2) * inv_r, dj_t, dz * inv_r, -e * kLn2);
+                            store_sample(a, set0 + n_feat, c, sqrt_approx(d2) * inv_r, dj_t, dz * inv_r, e * kLn2);
                             ++n_feat;
                         }
                         acc_r = fmaf(w, er, acc_r);
                         acc_g = fmaf(w, eg, acc_g);
                         acc_b = fmaf(w, eb, acc_b);
                         acc_w += w;
-                        ++n_acc;
+                        n_acc += 1.0f;
                     }
                 }
             }
@@ -516,11 +681,11 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
             // per pixel: the count kept, c_ref and the size of the whole set / 64 (what the plain
             // fallback averages)
             a.sets.n[crop_idx] = n_feat;
-            a.sets.info[crop_idx] = make_float4(cref.x, cref.y, cref.z, (float)n_acc * (1.0f / 64.0f));
+            a.sets.info[crop_idx] = make_float4(cref.x, cref.y, cref.z, n_acc * (1.0f / 64.0f));
         }
         if (DEBUG && a.pixel_stats) {
             int32_t *ps = a.pixel_stats + crop_idx * 3;
-            ps[0] = n_acc;
+            ps[0] = (int)n_acc;
             ps[1] = n_exam;
             ps[2] = __float_as_int(acc_w);
         }
@@ -560,8 +725,8 @@ __global__ void __launch_bounds__(kThreads, MINB) gather_kernel(const GatherArgs
         // the shutter weight of Eq. 10 replaces Eq. 4: no colour and no position term
         const bool shutter = a.mode == SSVP_MODE_SHUTTER;
         s_const[0] = r * r;
-        s_const[1] = shutter ? 0.0f : kLog2e / (2.0f * a.sigma_rgb * a.sigma_rgb);
-        s_const[2] = shutter ? 0.0f : kLog2e / (2.0f * sx * sx);
+        s_const[1] = shutter ? 0.0f : -kLog2e / (2.0f * a.sigma_rgb * a.sigma_rgb);
+        s_const[2] = shutter ? 0.0f : -kLog2e / (2.0f * sx * sx);
         s_const[3] = a.mode == SSVP_MODE_MEAN ? 0.0f : 1.0f;
     }
     __syncthreads();
@@ -570,9 +735,9 @@ __global__ void __launch_bounds__(kThreads, MINB) gather_kernel(const GatherArgs
     const int u = u0 + tx, v = v0 + ty;
     const bool active = u < a.x0 + a.cw && v < a.y0 + a.ch;
     const long long crop_idx = (long long)(v - a.y0) * a.cw + (u - a.x0);
-    int n_acc = 0, n_exam = 0;
-    float acc_w = 0.0f;
-    gather_pixel<K, CFMT, DEBUG, LEARN, 2, STG>(a, a.clip, O, u0, v0, u, v, active, crop_idx, sgeom, a.n_slots,
+    int n_exam = 0;
+    float n_acc = 0.0f, acc_w = 0.0f;
+    gather_pixel<K, CFMT, CFMT == 0 || LEARN ? 3 : 2, DEBUG, LEARN, STG>(a, a.clip, O, u0, v0, u, v, active, crop_idx, sgeom, a.n_slots,
                                                 s_const[0], s_const[1], s_const[2], s_const[3] != 0.0f, n_acc, n_exam,
                                                 acc_w, &tmap);
 
@@ -646,8 +811,8 @@ __global__ void __launch_bounds__(32 * TY, 32 / TY) batch_kernel(const GatherArg
                 const float r = a.radius > 0.0f ? a.radius : -a.radius * *b.clip[c].p.median;
                 const float sx = a.sigma_xyz > 0.0f ? a.sigma_xyz : r;
                 s_const[0] = r * r;
-                s_const[1] = kLog2e / (2.0f * a.sigma_rgb * a.sigma_rgb);
-                s_const[2] = kLog2e / (2.0f * sx * sx);
+                s_const[1] = -kLog2e / (2.0f * a.sigma_rgb * a.sigma_rgb);
+                s_const[2] = -kLog2e / (2.0f * sx * sx);
                 s_const[3] = a.mode == 3 ? 0.0f : 1.0f;
             }
         }
@@ -661,9 +826,9 @@ __global__ void __launch_bounds__(32 * TY, 32 / TY) batch_kernel(const GatherArg
         __syncthreads();
         const int u = u0 + (threadIdx.x & 31), v = v0 + (threadIdx.x >> 5);
         const bool active = u < bc.p.W && v < bc.p.H;
-        int n_acc = 0, n_exam = 0;
-        float acc_w = 0.0f;
-        gather_pixel<K, CFMT, false, false, 2>(a, bc.p, bc.frame_begin + oi, u0, v0, u, v, active, 0, sgeom, a.n_slots,
+        int n_exam = 0;
+        float n_acc = 0.0f, acc_w = 0.0f;
+        gather_pixel<K, CFMT, 2, false>(a, bc.p, bc.frame_begin + oi, u0, v0, u, v, active, 0, sgeom, a.n_slots,
                                                s_const[0], s_const[1], s_const[2], s_const[3] != 0.0f, n_acc, n_exam,
                                                acc_w);
         // launch statistics go to per-warp shared slots after every tile
@@ -764,9 +929,7 @@ cudaError_t launch_k(const GatherArgs &a, cudaStream_t s) {
             return cudaErrorInvalidValue;
         }
     }
-    if (a.sets.col && a.n_slots <= kLearnShortSlots)
-        gather_kernel<K, CFMT, false, true, kLearnCtasShort><<<grid, kThreads, smem, s>>>(a, tmap);
-    else if (a.sets.col) gather_kernel<K, CFMT, false, true><<<grid, kThreads, smem, s>>>(a, tmap);
+    if (a.sets.col) gather_kernel<K, CFMT, false, true, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
     else if (dbg) gather_kernel<K, CFMT, true><<<grid, kThreads, smem, s>>>(a, tmap);
     else gather_kernel<K, CFMT, false><<<grid, kThreads, smem, s>>>(a, tmap);
     return cudaGetLastError();

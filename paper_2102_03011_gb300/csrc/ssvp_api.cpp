@@ -589,10 +589,21 @@ void free_sets(ssvp::SampleSets &S) {
     S = ssvp::SampleSets{};
 }
 
-int learned_scratch(ssvp_ctx *ctx, size_t n_px) {
-    // the kernels address a crop's sets with one 32-bit sample index (pixel * 64 + slot)
+// the kernels address a crop's sets with one 32-bit sample index (pixel * 64 + slot)
+int learned_limit(ssvp_ctx *ctx, size_t n_px) {
     if (n_px * 64 > 0xffffffffull)
         return fail(ctx, SSVP_EINVAL, "the learned filter takes crops of at most 67,108,863 pixels (have %zu)", n_px);
+    return SSVP_OK;
+}
+
+// Whether a training batch of n_batch pixels of an n_px-pixel frame is extracted by the list (one warp a
+// pixel) or with the whole frame: a listed pixel costs about four times a pixel of the frame (640 x 360,
+// +-15: 131 us for 16,384 listed pixels, 385 us for the frame's 230,400; at 60,000 pixels a gradient takes
+// 0.88 ms either way).
+bool batch_by_list(size_t n_batch, size_t n_px) { return 4 * n_batch < n_px; }
+
+int learned_scratch(ssvp_ctx *ctx, size_t n_px) {
+    if (int rc = learned_limit(ctx, n_px); rc != SSVP_OK) return rc;
     if (n_px <= ctx->l_cap) return SSVP_OK;
     CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
     free_sets(ctx->l_sets);
@@ -607,8 +618,10 @@ int learned_scratch(ssvp_ctx *ctx, size_t n_px) {
     return SSVP_OK;
 }
 
-// capped sample sets of output frame O of a clip over a crop, into the context's scratch
-int extract_samples(ssvp_ctx *ctx, const ssvp_params &p, int clip_id, int O, int x0, int y0, int cw, int ch) {
+// capped sample sets of output frame O of a clip over a crop, into the context's scratch; with a list
+// (n_list pixels v * W + u on the device; the crop is the whole frame) only of the listed pixels
+int extract_samples(ssvp_ctx *ctx, const ssvp_params &p, int clip_id, int O, int x0, int y0, int cw, int ch,
+                    const int32_t *list = nullptr, int n_list = 0) {
     Clip &c = ctx->clips[clip_id];
     const int T = p.half_window, ns = 2 * T + 1;
     if ((size_t)ns > ctx->geom_cap) {
@@ -641,7 +654,8 @@ int extract_samples(ssvp_ctx *ctx, const ssvp_params &p, int clip_id, int O, int
     a.stat_counts = ctx->stat_counts;
     a.stat_sumw = ctx->stat_sumw;
     TraceScope ts(ctx, SSVP_TRACE_EXTRACT, ctx->stream);
-    CK(ssvp::launch_gather(a, ctx->stream), "gather kernel (learned samples)");
+    if (list) CK(ssvp::launch_extract_list(a, list, n_list, ctx->stream), "list extraction kernel (learned samples)");
+    else CK(ssvp::launch_gather(a, ctx->stream), "gather kernel (learned samples)");
     return SSVP_OK;
 }
 
@@ -1759,7 +1773,9 @@ int ssvp_mlp_grad(ssvp_ctx *ctx, const ssvp_params *params, int clip_id, const i
     for (int i = 0; i < n_pixels; ++i)
         if (pixels[i] < 0 || (size_t)pixels[i] >= npx) return fail(ctx, SSVP_EINVAL, "pixel index out of range");
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
-    if ((rc = learned_scratch(ctx, npx)) != SSVP_OK) return rc;
+    const bool by_list = batch_by_list((size_t)n_pixels, npx);
+    if ((rc = learned_limit(ctx, npx)) != SSVP_OK) return rc;
+    if ((rc = learned_scratch(ctx, by_list ? (size_t)n_pixels : npx)) != SSVP_OK) return rc;
     if ((size_t)n_pixels > ctx->l_batch_cap) {
         CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
         if (ctx->l_batch) cudaFree(ctx->l_batch);
@@ -1767,9 +1783,9 @@ int ssvp_mlp_grad(ssvp_ctx *ctx, const ssvp_params *params, int clip_id, const i
         CK(cudaMalloc(&ctx->l_batch, n_pixels * sizeof(int32_t)), "cudaMalloc (batch)");
         ctx->l_batch_cap = n_pixels;
     }
-    if ((rc = extract_samples(ctx, *params, clip_id, O, 0, 0, c.p.W, c.p.H)) != SSVP_OK)
-        return rc;
     CK(cudaMemcpyAsync(ctx->l_batch, pixels, n_pixels * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream), "cudaMemcpyAsync");
+    if ((rc = extract_samples(ctx, *params, clip_id, O, 0, 0, c.p.W, c.p.H, by_list ? ctx->l_batch : nullptr, n_pixels)) != SSVP_OK)
+        return rc;
     CK(cudaMemsetAsync(ctx->mlp.grad, 0, (ssvp::kMlpParams + 1) * sizeof(float), ctx->stream), "cudaMemsetAsync");
     ssvp::MlpArgs m{};
     m.w = mlp_weights(ctx);
@@ -1778,6 +1794,7 @@ int ssvp_mlp_grad(ssvp_ctx *ctx, const ssvp_params *params, int clip_id, const i
     m.O = O; m.W = c.p.W; m.H = c.p.H; m.x0 = 0; m.y0 = 0; m.cw = c.p.W;
     m.batch = ctx->l_batch;
     m.n_batch = n_pixels;
+    m.sets_by_batch = by_list;
     m.clean = clean;
     m.bce_w = 0.1f;
     m.grad = ctx->mlp.grad;
@@ -1800,7 +1817,7 @@ int ssvp_train(ssvp_ctx *ctx, const ssvp_params *params, const int *clip_ids, co
     if (!clip_ids || !clean || n_clips < 1) return fail(ctx, SSVP_EINVAL, "bad clip list");
     if (params->k > 7) return fail(ctx, SSVP_EINVAL, "the learned filter supports k <= 7");
     if (loss_out && (rc = check_mem(ctx, loss_out, SSVP_MEM_HOST, "loss_out")) != SSVP_OK) return rc;
-    size_t max_px = 0;
+    size_t max_px = 0, max_sets = 0;
     for (int i = 0; i < n_clips; ++i) {
         if (clip_ids[i] < 0 || clip_ids[i] >= SSVP_MAX_CLIPS) return fail(ctx, SSVP_EINVAL, "clip_id out of range");
         const Clip &c = ctx->clips[clip_ids[i]];
@@ -1808,7 +1825,9 @@ int ssvp_train(ssvp_ctx *ctx, const ssvp_params *params, const int *clip_ids, co
         if (!c.has_cams) return fail(ctx, SSVP_ENOCAM, "clip %d has no cameras", clip_ids[i]);
         if (!clean[i]) return fail(ctx, SSVP_EINVAL, "clean target of clip %d is NULL", clip_ids[i]);
         if ((rc = check_mem(ctx, clean[i], SSVP_MEM_DEVICE, "clean target")) != SSVP_OK) return rc;
-        max_px = std::max(max_px, (size_t)c.p.W * c.p.H);
+        const size_t npx = (size_t)c.p.W * c.p.H, nb = (size_t)cfg->batch_pixels;
+        max_px = std::max(max_px, npx);
+        max_sets = std::max(max_sets, batch_by_list(nb, npx) ? nb : npx);
     }
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
     if ((rc = mlp_alloc(ctx)) != SSVP_OK) return rc;
@@ -1820,7 +1839,8 @@ int ssvp_train(ssvp_ctx *ctx, const ssvp_params *params, const int *clip_ids, co
         for (auto &x : W2) x = (float)(rng.normal() * std::sqrt(2.0 / 64.0));
         if ((rc = ssvp_set_mlp(ctx, W1.data(), b1.data(), W2.data(), b2.data())) != SSVP_OK) return rc;
     }
-    if ((rc = learned_scratch(ctx, max_px)) != SSVP_OK) return rc;
+    if ((rc = learned_limit(ctx, max_px)) != SSVP_OK) return rc;
+    if ((rc = learned_scratch(ctx, max_sets)) != SSVP_OK) return rc;
     const size_t nb = (size_t)cfg->batch_pixels;
     if (nb > ctx->l_batch_cap) {
         CK(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
@@ -1843,11 +1863,13 @@ int ssvp_train(ssvp_ctx *ctx, const ssvp_params *params, const int *clip_ids, co
         const int O = (int)(rng.next() % (uint64_t)c.p.F);
         const uint64_t npx = (uint64_t)c.p.W * c.p.H;
         for (auto &b : batch) b = (int32_t)(rng.next() % npx);
-        if ((rc = extract_samples(ctx, *params, clip_ids[ci], O, 0, 0, c.p.W, c.p.H)) != SSVP_OK)
-            return rc;
         // pageable source: the copy is staged before the call returns, so batch may be rewritten
         CK(cudaMemcpyAsync(ctx->l_batch, batch.data(), nb * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream),
            "cudaMemcpyAsync");
+        const bool by_list = batch_by_list(nb, (size_t)npx);
+        if ((rc = extract_samples(ctx, *params, clip_ids[ci], O, 0, 0, c.p.W, c.p.H, by_list ? ctx->l_batch : nullptr,
+                                  (int)nb)) != SSVP_OK)
+            return rc;
         CK(cudaMemsetAsync(ctx->mlp.grad, 0, (ssvp::kMlpParams + 1) * sizeof(float), ctx->stream), "cudaMemsetAsync");
         ssvp::MlpArgs m{};
         m.w = mlp_weights(ctx);
@@ -1856,6 +1878,7 @@ int ssvp_train(ssvp_ctx *ctx, const ssvp_params *params, const int *clip_ids, co
         m.O = O; m.W = c.p.W; m.H = c.p.H; m.x0 = 0; m.y0 = 0; m.cw = c.p.W;
         m.batch = ctx->l_batch;
         m.n_batch = (long long)nb;
+        m.sets_by_batch = by_list;
         m.clean = clean[ci];
         m.bce_w = cfg->bce_weight;
         m.grad = ctx->mlp.grad;

@@ -146,6 +146,7 @@ struct MlpArgs {
     float *out;                   // clip output buffer (inference)
     float *conf_out;              // optional per crop pixel confidence
     const int32_t *batch;         // training: crop pixel indices
+    int sets_by_batch;            // training: the sets are stored by batch position, not by crop pixel
     long long n_batch;
     const float *clean;           // training: target frames (F x H x W x 3, FP32)
     float bce_w;
@@ -170,6 +171,8 @@ cudaError_t launch_pack(const float *rgb, const float *depth, int W, int H, int 
 cudaError_t launch_median(const Planes &p, unsigned int *scratch, cudaStream_t s);
 size_t median_scratch_words();
 cudaError_t launch_gather(const GatherArgs &a, cudaStream_t s);
+// capped sample sets of the listed pixels (v * W + u) of frame a.frame_begin, stored by list position
+cudaError_t launch_extract_list(const GatherArgs &a, const int32_t *list, int n_list, cudaStream_t s);
 cudaError_t launch_aperture(const GatherArgs &a, cudaStream_t s);
 cudaError_t launch_frustum(const GatherArgs &a, cudaStream_t s);
 cudaError_t launch_grad_sum(const Planes &p, cudaStream_t s);

@@ -547,14 +547,15 @@ __global__ void __launch_bounds__(kTcThreads, 3) mlp_train_tc_kernel(const MlpAr
         float pl[3] = {0.f, 0.f, 0.f};
         if (bi < m.n_batch) {
             px = m.batch[bi];
-            n = m.sets.n[px];
-            const long long k = px * kS + srow;
+            const long long si = m.sets_by_batch ? bi : px;
+            n = m.sets.n[si];
+            const long long k = si * kS + srow;
             c = __ldg(m.sets.col + k);
             f89 = __ldg(m.sets.f89 + k);
-            info = __ldg(m.sets.info + px);
-            pl[0] = m.sets.plain[3 * px];
-            pl[1] = m.sets.plain[3 * px + 1];
-            pl[2] = m.sets.plain[3 * px + 2];
+            info = __ldg(m.sets.info + si);
+            pl[0] = m.sets.plain[3 * si];
+            pl[1] = m.sets.plain[3 * si + 1];
+            pl[2] = m.sets.plain[3 * si + 2];
         }
         const bool valid = srow < n;
         // 2. features (logical order; slot 15 carries 1.0 for b1 in the layer-1 operand only)

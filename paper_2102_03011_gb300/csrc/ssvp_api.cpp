@@ -56,6 +56,7 @@ void swap_window(Planes &a, Planes &b) {
     std::swap(a.colour, b.colour);
     std::swap(a.median, b.median);
     std::swap(a.zrange, b.zrange);
+    std::swap(a.tiles, b.tiles);
     std::swap(a.grad_sum, b.grad_sum);
     std::swap(a.grad_log2, b.grad_log2);
     std::swap(a.grad_partial, b.grad_partial);
@@ -825,13 +826,14 @@ int ssvp_load_clip(ssvp_ctx *ctx, int clip_id, int W, int H, int F, const float 
         (e = cudaMalloc(&p.colour, nplane * texel)) != cudaSuccess ||
         (e = cudaMalloc(&p.out, nout * sizeof(float))) != cudaSuccess ||
         (e = cudaMalloc(&p.median, sizeof(float))) != cudaSuccess ||
-        (e = cudaMalloc(&p.zrange, 2 * sizeof(unsigned int) * (size_t)F)) != cudaSuccess ||
+        (e = cudaMalloc(&p.zrange, ssvp::zrange_bytes(W, H, F))) != cudaSuccess ||
         (e = cudaMalloc(&p.grad_sum, sizeof(double) * (size_t)F)) != cudaSuccess ||
         (e = cudaMalloc(&p.grad_log2, sizeof(float) * (size_t)F)) != cudaSuccess ||
         (e = cudaMalloc(&p.grad_partial, sizeof(double) * ssvp::grad_partial_words(F))) != cudaSuccess)) {
         free_clip(c);
         return cuda_fail(ctx, e, "cudaMalloc (clip planes)");
     }
+    p.tiles = (float2 *)((char *)p.zrange + ssvp::zrange_tiles_offset(F));
     // the load's work goes to the high-priority load stream, after everything already queued on
     // the context's stream (which may still read the planes being replaced)
     cudaStream_t ls = ctx->load_stream;
@@ -982,7 +984,7 @@ int ssvp_append_frames(ssvp_ctx *ctx, int clip_id, int n, const float *rgb, cons
         if ((e = cudaMalloc(&sp.depth, nplane * sizeof(float))) != cudaSuccess ||
             (e = cudaMalloc(&sp.colour, nplane * texel)) != cudaSuccess ||
             (e = cudaMalloc(&sp.median, sizeof(float))) != cudaSuccess ||
-            (e = cudaMalloc(&sp.zrange, 2 * sizeof(unsigned int) * (size_t)F)) != cudaSuccess ||
+            (e = cudaMalloc(&sp.zrange, ssvp::zrange_bytes(W, H, F))) != cudaSuccess ||
             (e = cudaMalloc(&sp.grad_sum, sizeof(double) * (size_t)F)) != cudaSuccess ||
             (e = cudaMalloc(&sp.grad_log2, sizeof(float) * (size_t)F)) != cudaSuccess ||
             (e = cudaMalloc(&sp.grad_partial, sizeof(double) * ssvp::grad_partial_words(F))) != cudaSuccess ||
@@ -993,6 +995,7 @@ int ssvp_append_frames(ssvp_ctx *ctx, int clip_id, int n, const float *rgb, cons
             sp = Planes{};
             return cuda_fail(ctx, e, "cudaMalloc (spare window)");
         }
+        sp.tiles = (float2 *)((char *)sp.zrange + ssvp::zrange_tiles_offset(F));
         CK(cudaMemsetAsync(sp.depth, 0xff, nplane * sizeof(float), ctx->stream), "cudaMemsetAsync");
         CK(cudaMemsetAsync(sp.colour, 0, nplane * texel, ctx->stream), "cudaMemsetAsync");
         CK(cudaEventRecord(c.ev_append, ctx->stream), "cudaEventRecord");
@@ -1009,6 +1012,7 @@ int ssvp_append_frames(ssvp_ctx *ctx, int clip_id, int n, const float *rgb, cons
     q.colour = sp.colour;
     q.median = sp.median;
     q.zrange = sp.zrange;
+    q.tiles = sp.tiles;
     q.grad_sum = sp.grad_sum;
     q.grad_log2 = sp.grad_log2;
     q.grad_partial = sp.grad_partial;

@@ -25,6 +25,8 @@ struct Planes {
     float *median;         // device scalar: lower-median valid depth
     unsigned int *zrange;  // F x 2 words: valid depth range of each frame as bit patterns,
                            // complement of the minimum's bits and the maximum's bits (0: none)
+    float2 *tiles;         // F x tile rows x tile columns: valid depth range (min, max) of each 8 x 8 pixel tile,
+                           // (inf, 0) without one; in zrange's allocation, computed with it
     double *grad_sum;      // F: Eq. 5 blurriness measure (sum of gradient magnitudes) per frame
     float *grad_log2;      // F: log2(grad_sum / max over frames), the Eq. 5 factor in log2 units
     double *grad_partial;  // F x grad_partial_words(1): partial sums of grad_sum
@@ -179,6 +181,11 @@ cudaError_t launch_grad_sum(const Planes &p, cudaStream_t s);
 cudaError_t launch_mask_box(const Planes &p, const double *cam, const double *box, cudaStream_t s);
 size_t grad_partial_words(int F);
 cudaError_t launch_zrange(const Planes &p, cudaStream_t s);
+// bytes of the zrange allocation, which holds the tiles after the frames' words, and the tiles' offset in it
+inline size_t zrange_tiles_offset(int F) { return (2 * sizeof(unsigned int) * (size_t)F + 255) / 256 * 256; }
+inline size_t zrange_bytes(int W, int H, int F) {
+    return zrange_tiles_offset(F) + sizeof(float) * 2 * (size_t)F * (size_t)((W + 7) / 8) * (size_t)((H + 7) / 8);
+}
 // persistent batched gather; grid = batch_grid(...) CTAs
 cudaError_t launch_batch(const GatherArgs &a, const BatchArgs &b, int tile_rows, int colour_fmt, int grid,
                          cudaStream_t s);

@@ -185,8 +185,8 @@ constexpr int kTile = 8;       // side of the depth range tiles
 template <bool SR> constexpr int kLongHull = SR ? 48 : 32;
 constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: x + kRound holds x rounded to an integer in its low bits
 
-// S: each pixel's window slots are shared out to S threads (the CTA takes 32 x 8 / S pixels), which join
-// their sums after each pass
+// S (a power of two): each pixel's window frames are shared out to S threads (the CTA takes 32 x 8 / S pixels),
+// by J modulo S, whatever the window; they join their sums after each pass
 template <int CFMT, bool DEBUG, bool SR, int INP, int S>
 __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const GatherArgs a) {
     constexpr int kRows = kFrTileY / S;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
     acc_r = acc_g = acc_b = acc_w = 0.0f;
     m_log2 = wpass ? kNoWeight : 0.0f;
     if (gather) {
-        for (int j = split; j < ns; j += S) {
+        for (int j = (split - (O - a.T)) & (S - 1); j < ns; j += S) {
             const float4 *sl = s_slot + kFrSlotVec * j;
             const float4 q3 = sl[3];
             const int J = __float_as_int(q3.w);

@@ -101,16 +101,16 @@ __device__ __forceinline__ unsigned stg_box(const float4 *sgeom, int n_slots, in
 }
 __device__ __forceinline__ unsigned stg_bar(int b) { return smem_addr(&g_stg_bar[threadIdx.x >> 5][b]); }
 
-// Issue the copy of window slot s (frame J) into buffer s & 1: called by the warp's first gathering
+// Issue the copy of window slot s (frame J), the seq-th in the warp's order, into buffer seq & 1: called by the warp's first gathering
 // lane, whose pixel offset in the tile is (du, dv), depth dref and lane index `lane`; tmap describes
 // the clip's depth planes ({pitch, rows, F} floats, box {kBoxW, kBoxH, 1}).  skip (a test of the
 // time-out path): the barrier is told to expect the box's bytes but no copy is issued, so the wait
 // for it runs out.
 template <int K>
-__device__ __forceinline__ void stage_issue(const CUtensorMap *tmap, const float4 *sgeom, int n_slots, int s, float du,
+__device__ __forceinline__ void stage_issue(const CUtensorMap *tmap, const float4 *sgeom, int n_slots, int s, int seq, float du,
                                             float dv, float dref, int lane, bool skip) {
     constexpr int h = (K - 1) / 2;
-    const int b = s & 1;
+    const int b = seq & 1;
     const float4 *g = sgeom + kSlotVec * s;
     const int J = __float_as_int(g[5].w);
     int x0 = kNoBox, y0 = kNoBox;
@@ -146,6 +146,17 @@ __device__ __forceinline__ void stage_issue(const CUtensorMap *tmap, const float
     } else {
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
     }
+}
+
+// The slot after jj in the order by groups ((group0 + jj) mod 4 rising, then jj); jj = -4: the first slot; -1
+// after the last
+__device__ __forceinline__ int next_slot(int jj, int group0, int n_slots) {
+    if (jj >= 0 && jj + 4 < n_slots) return jj + 4;
+    for (int g = jj < 0 ? 0 : ((group0 + jj) & 3) + 1; g < 4; ++g) {
+        const int first = (g - group0) & 3;
+        if (first < n_slots) return first;
+    }
+    return -1;
 }
 
 // The gather and filter of one output pixel (u, v) of frame O (steps A3-A7).  sgeom holds the
@@ -361,16 +372,21 @@ __device__ __forceinline__ void window_centre(const df U, const df V, float &cxf
 // STG: the candidate depths of the test loop come from the warp's staged boxes (K > 0, not LEARN);
 // tmap describes the clip's depth planes
 // a_rgb and a_xyz: -log2(e) / (2 sigma^2) of Eq. 4's colour and position terms
+// The window's frames are summed in four groups, by J modulo 4 whatever the window, each from zero and in
+// order, and the groups' sums are added in order (LEARN: in one group, canonical order).  S = 1: this thread
+// goes through all four; S = 4: the pixel has four threads of the CTA, this one taking group `split`.  The
+// result is the same to the bit.  s_sum: 4 x NT floats of shared memory for the groups' sums; NT threads a CTA.
 // NS: survivors per iteration of the filter loop of a compile-time window.  Each is one more record in
 // flight and up to NS - 1 idle slots at the end of a frame's list: 2 -> 3 takes a 1080p +-30 FP32 frame
 // from 4.15 to 3.99 ms, but with FP16 colour, whose samples take two loads and conversions, and in the
 // batched kernel the registers run out (a 720p FP16 frame 1.03 -> 1.06 ms, the mixed clips' plan 13.5 -> 14.0)
-template <int K, int CFMT, int NS, bool DEBUG, bool LEARN = false, bool STG = false>
+template <int K, int CFMT, int NS, int NT, bool DEBUG, bool LEARN = false, bool STG = false, int S = 1>
 __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &P, const int O, const int u0,
                                              const int v0, const int u, const int v, const bool active,
                                              const long long crop_idx, const float4 *sgeom, const int n_slots,
                                              const float r2, const float a_rgb, const float a_xyz, const bool weighted,
-                                             float &n_acc, int &n_exam, float &acc_w, const CUtensorMap *tmap = nullptr) {
+                                             float &n_acc, int &n_exam, float &acc_w, float *s_sum, const int split = 0,
+                                             const CUtensorMap *tmap = nullptr) {
     static_assert(!STG || (K > 0 && K <= kStageMaxK && !LEARN), "staging: compile-time k <= 7, plain gather");
     using WB = WindowBits<K>;
     constexpr int kTestRows = K == 7 && (NS == 2 || LEARN) ? 2 : 1;  // see test_distance
@@ -412,22 +428,41 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
 
     if (gather) {
         const float du = (float)(u - u0), dv = (float)(v - v0);
+        const int group0 = O - Tw;  // slot jj belongs to group (group0 + jj) mod 4
+        int n_seen = 0;                         // STG: slots so far (slot n_seen is in buffer n_seen & 1)
         if (STG && (int)(threadIdx.x & 31) == __ffs(G) - 1)
-            stage_issue<K>(tmap, sgeom, n_slots, 0, du, dv, dref, threadIdx.x & 31, a.stage == 2);
-        for (int jj = 0; jj < n_slots; ++jj) {
+            stage_issue<K>(tmap, sgeom, n_slots, next_slot(-4, group0, n_slots), 0, du, dv, dref, threadIdx.x & 31, a.stage == 2);
+        // S = 1: a finished group's sums join those before it, in shared memory (in registers they spill)
+        float *sum = LEARN ? nullptr : s_sum + (S > 1 ? split * NT + threadIdx.x % (NT / S) : threadIdx.x);
+        constexpr int kStride = NT / S;
+        if (!LEARN && S == 1) sum[0] = sum[kStride] = sum[2 * kStride] = sum[3 * kStride] = 0.0f;
+        auto following = [&](int jj) {
+            if (LEARN) return jj + 1;
+            if (S > 1 || jj + 4 < n_slots) return jj + 4;
+            sum[0] += acc_r;
+            sum[kStride] += acc_g;
+            sum[2 * kStride] += acc_b;
+            sum[3 * kStride] += acc_w;
+            acc_r = acc_g = acc_b = acc_w = 0.0f;
+            const int nx = next_slot(jj, group0, n_slots);
+            return nx < 0 ? n_slots : nx;
+        };
+        for (int jj = LEARN ? 0 : S > 1 ? (split - group0) & 3 : next_slot(-4, group0, n_slots); jj < n_slots;
+             jj = following(jj), ++n_seen) {
             int2 org = make_int2(kNoBox, kNoBox);
             if (STG) {
-                // every lane of G is done with buffer (jj + 1) & 1 (slot jj - 1): refill it with slot
-                // jj + 1, then wait for slot jj
+                // every lane of G is done with the other buffer (the slot before): refill it with the next
+                // slot, then wait for this one
                 __syncwarp(G);
                 const bool leader = (int)(threadIdx.x & 31) == __ffs(G) - 1;
-                if (stg_fail < 0 && leader && jj + 1 < n_slots)
-                    stage_issue<K>(tmap, sgeom, n_slots, jj + 1, du, dv, dref, threadIdx.x & 31, a.stage == 2);
-                const bool ok = stg_fail >= 0 || stg_wait(stg_bar(jj & 1), (unsigned)(jj >> 1) & 1u);
+                if (stg_fail < 0 && leader && n_seen + 1 < n_slots)
+                    stage_issue<K>(tmap, sgeom, n_slots, next_slot(jj, group0, n_slots), n_seen + 1, du, dv, dref,
+                                   threadIdx.x & 31, a.stage == 2);
+                const bool ok = stg_fail >= 0 || stg_wait(stg_bar(n_seen & 1), (unsigned)(n_seen >> 1) & 1u);
                 if (__all_sync(G, ok)) {
-                    if (stg_fail < 0) org = g_stg_org[threadIdx.x >> 5][jj & 1];
+                    if (stg_fail < 0) org = g_stg_org[threadIdx.x >> 5][n_seen & 1];
                 } else if (stg_fail < 0) {
-                    stg_fail = jj;  // the rest of this warp's frames test from the global plane
+                    stg_fail = n_seen;  // the rest of this warp's frames test from the global plane
                     if (leader) atomicOr(a.err, 2);
                 }
             }
@@ -497,7 +532,7 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
                     if ((unsigned)ox <= (unsigned)(kBoxW - K) && (unsigned)oy <= (unsigned)(kBoxH - K)) {
                         // box columns start at a multiple of four, so ox has the parity of xw
                         dtest = reinterpret_cast<const float *>(reinterpret_cast<const char *>(sgeom) +
-                                                                (stg_box(sgeom, n_slots, jj & 1) - smem_addr(sgeom))) +
+                                                                (stg_box(sgeom, n_slots, n_seen & 1) - smem_addr(sgeom))) +
                                 oy * kBoxW + (ox - par);
                         tpitch = kBoxW;
                     }
@@ -664,6 +699,12 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
                 }
             }
         }
+        if (!LEARN && S > 1) {
+            sum[0] = acc_r;
+            sum[kStride] = acc_g;
+            sum[2 * kStride] = acc_b;
+            sum[3 * kStride] = acc_w;
+        }
         if (STG && stg_fail >= 0 && (int)(threadIdx.x & 31) == __ffs(G) - 1) {
             // after a time-out: wait once more (bounded) for the copies that may still be in flight,
             // slot stg_fail and the slot issued before its wait
@@ -672,6 +713,34 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
         }
     }
 
+    if (!LEARN && S == 1 && gather) {
+        acc_r = s_sum[threadIdx.x];
+        acc_g = s_sum[NT + threadIdx.x];
+        acc_b = s_sum[2 * NT + threadIdx.x];
+        acc_w = s_sum[3 * NT + threadIdx.x];
+    }
+    if constexpr (S > 1) {
+        __syncthreads();
+        if (split != 0) {
+            acc_w = 0.0f;  // counted with the first thread's in the launch statistics
+            return;
+        }
+        if (gather) {
+            constexpr int kStride = NT / S;
+            const float *sum = s_sum + threadIdx.x % kStride;
+            acc_r = sum[0];
+            acc_g = sum[kStride];
+            acc_b = sum[2 * kStride];
+            acc_w = sum[3 * kStride];
+#pragma unroll
+            for (int s = 1; s < S; ++s) {
+                acc_r = sum[s * NT] + acc_r;
+                acc_g = sum[s * NT + kStride] + acc_g;
+                acc_b = sum[s * NT + 2 * kStride] + acc_b;
+                acc_w = sum[s * NT + 3 * kStride] + acc_w;
+            }
+        }
+    }
     if (active) {
         // Eq. 3 written around the reference colour: c_ref + sum w (c - c_ref) / sum w
         float o_r = cref.x, o_g = cref.y, o_b = cref.z;
@@ -704,7 +773,7 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
 // One CTA per 32 x kTileY output tile of one output frame (grid: tiles x output frames).
 // STG: the staged gather; dynamic shared memory then holds, after the slot geometry (aligned up to
 // 128 bytes), two boxes per warp, and tmap describes the clip's depth planes.
-template <int K, int CFMT, bool DEBUG, bool LEARN = false, int MINB = SSVP_MIN_CTAS, bool STG = false>
+template <int K, int CFMT, bool DEBUG, bool LEARN = false, int MINB = SSVP_MIN_CTAS, bool STG = false, int S = 1>
 __global__ void __launch_bounds__(kThreads, MINB) gather_kernel(const GatherArgs a, const __grid_constant__ CUtensorMap tmap) {
     extern __shared__ float4 sgeom[];
     __shared__ float s_const[4];
@@ -718,7 +787,9 @@ __global__ void __launch_bounds__(kThreads, MINB) gather_kernel(const GatherArgs
 
     const int oi = blockIdx.z;
     const int O = a.frame_begin + oi;
-    const int u0 = a.x0 + blockIdx.x * kTileX, v0 = a.y0 + blockIdx.y * kTileY;
+    constexpr int kRows = kTileY / S;
+    // the geometry is that of the kTileY-row tile the rows lie in, whatever S (its rounding decides ties)
+    const int u0 = a.x0 + blockIdx.x * kTileX, vt = blockIdx.y * kRows, v0 = a.y0 + vt / kTileY * kTileY;
     for (int j = threadIdx.x; j < a.n_slots; j += kThreads) {
         float4 *g = sgeom + kSlotVec * j;
         build_slot(a.geom[(long long)oi * a.n_slots + j], (float)u0, (float)v0, g);
@@ -739,15 +810,16 @@ __global__ void __launch_bounds__(kThreads, MINB) gather_kernel(const GatherArgs
     }
     __syncthreads();
 
-    const int tx = threadIdx.x % kTileX, ty = threadIdx.x / kTileX;
-    const int u = u0 + tx, v = v0 + ty;
+    const int tx = threadIdx.x % kTileX, ty = threadIdx.x / kTileX % kRows, split = threadIdx.x / (kTileX * kRows);
+    const int u = u0 + tx, v = a.y0 + vt + ty;
     const bool active = u < a.x0 + a.cw && v < a.y0 + a.ch;
     const long long crop_idx = (long long)(v - a.y0) * a.cw + (u - a.x0);
     int n_exam = 0;
     float n_acc = 0.0f, acc_w = 0.0f;
-    gather_pixel<K, CFMT, CFMT == 0 || LEARN ? 3 : 2, DEBUG, LEARN, STG>(a, a.clip, O, u0, v0, u, v, active, crop_idx, sgeom, a.n_slots,
-                                                s_const[0], s_const[1], s_const[2], s_const[3] != 0.0f, n_acc, n_exam,
-                                                acc_w, &tmap);
+    __shared__ float s_sum[LEARN ? 1 : 4 * kThreads];
+    gather_pixel<K, CFMT, CFMT == 0 || LEARN ? 3 : 2, kThreads, DEBUG, LEARN, STG, S>(
+        a, a.clip, O, u0, v0, u, v, active, crop_idx, sgeom, a.n_slots, s_const[0], s_const[1], s_const[2], s_const[3] != 0.0f,
+        n_acc, n_exam, acc_w, s_sum, split, &tmap);
 
     // launch statistics: warp, then block, then one atomic per CTA
     unsigned long long ce = (unsigned long long)n_exam, ca = (unsigned long long)n_acc;
@@ -786,6 +858,7 @@ __global__ void __launch_bounds__(32 * TY, 32 / TY) batch_kernel(const GatherArg
     __shared__ int s_c, s_u0, s_v0, s_oi, s_olast, s_done;
     __shared__ unsigned long long s_cnt[2][NT / 32];
     __shared__ double s_w[NT / 32];
+    __shared__ float s_sum[4 * NT];
     const int warp = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) { s_cnt[0][warp] = 0ull; s_cnt[1][warp] = 0ull; s_w[warp] = 0.0; }
     if (threadIdx.x == 0) { s_oi = 0; s_olast = 0; s_done = 0; }
@@ -836,9 +909,9 @@ __global__ void __launch_bounds__(32 * TY, 32 / TY) batch_kernel(const GatherArg
         const bool active = u < bc.p.W && v < bc.p.H;
         int n_exam = 0;
         float n_acc = 0.0f, acc_w = 0.0f;
-        gather_pixel<K, CFMT, 2, false>(a, bc.p, bc.frame_begin + oi, u0, v0, u, v, active, 0, sgeom, a.n_slots,
-                                               s_const[0], s_const[1], s_const[2], s_const[3] != 0.0f, n_acc, n_exam,
-                                               acc_w);
+        gather_pixel<K, CFMT, 2, NT, false>(a, bc.p, bc.frame_begin + oi, u0, v0, u, v, active, 0, sgeom, a.n_slots,
+                                            s_const[0], s_const[1], s_const[2], s_const[3] != 0.0f, n_acc, n_exam, acc_w,
+                                            s_sum);
         // launch statistics go to per-warp shared slots after every tile
         unsigned ce = (unsigned)n_exam, ca = (unsigned)n_acc;
         float sw = acc_w;
@@ -1090,7 +1163,22 @@ cudaError_t launch_k(const GatherArgs &a, cudaStream_t s) {
     }
     if (a.sets.col) gather_kernel<K, CFMT, false, true, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
     else if (dbg) gather_kernel<K, CFMT, true><<<grid, kThreads, smem, s>>>(a, tmap);
-    else gather_kernel<K, CFMT, false><<<grid, kThreads, smem, s>>>(a, tmap);
+    else {
+        // Few CTAs leave SMs idle or end in a nearly empty wave: below two and a half waves each pixel's frames
+        // are shared out to four threads (CTAs of 32 x 2 pixels).  One frame of 320 x 180, +-15 (0.4 waves):
+        // 104 -> 73 us; the 16 frames of 160 x 90 (1.6): 100 -> 96; 640 x 360 (1.5): 312 -> 261; six frames of
+        // 320 x 180 (2.3): 300 -> 275; two of 640 x 360, k = 5 (3.0): 351 against 360, one of 720p (5.9) 940 against 976.
+        // Each CTA builds the geometry of all frames, so above one wave only for windows of 16 frames and more
+        // (669 x 379, +-3, k = 3, 1.7 waves: 2 % slower shared out).
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        const long long ctas = (long long)grid.x * grid.y * grid.z, wave = (long long)SSVP_MIN_CTAS * sms;
+        if (ctas < wave || (2 * ctas < 5 * wave && a.n_slots >= 16)) {
+            grid.y = (a.ch + kTileY / 4 - 1) / (kTileY / 4);
+            gather_kernel<K, CFMT, false, false, SSVP_MIN_CTAS, false, 4><<<grid, kThreads, smem, s>>>(a, tmap);
+        } else gather_kernel<K, CFMT, false><<<grid, kThreads, smem, s>>>(a, tmap);
+    }
     return cudaGetLastError();
 }
 

@@ -599,8 +599,7 @@ int learned_limit(ssvp_ctx *ctx, size_t n_px) {
 
 // Whether a training batch of n_batch pixels of an n_px-pixel frame is extracted by the list (one warp a
 // pixel) or with the whole frame: a listed pixel costs about four times a pixel of the frame (640 x 360,
-// +-15: 131 us for 16,384 listed pixels, 385 us for the frame's 230,400; at 60,000 pixels a gradient takes
-// 0.88 ms either way).
+// +-15: 105 us for 16,384 listed pixels, 385 us for the frame's 230,400).
 bool batch_by_list(size_t n_batch, size_t n_px) { return 4 * n_batch < n_px; }
 
 int learned_scratch(ssvp_ctx *ctx, size_t n_px) {

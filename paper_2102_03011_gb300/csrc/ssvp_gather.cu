@@ -936,19 +936,22 @@ __global__ void __launch_bounds__(32 * TY, 32 / TY) batch_kernel(const GatherArg
 
 // Capped sample sets of a list of pixels of one frame (training batches): one warp a pixel, so that no
 // pixel outside the list is gathered.  The lanes first project the pixel into 32 window frames at once,
-// then take each frame's window together, lane = candidate (rows 0-3, then 4-6 of an 8-column grid), and
-// the accepted ones in lane order are the samples in canonical order.  The geometry is that of the tiles
+// then take each frame's window together, lane = candidate (rows 0-3, then 4-6 of an 8-column grid); the
+// accepted ones, in canonical order, queue up and are filtered 32 at a time.  The geometry is that of the tiles
 // of gather_kernel, so the sets are the same; the plain result's sums are per lane and differ in rounding.
-// Bound by instruction issue (0.65 of the slots) and the latency of the scattered window loads: 5,000 warp
-// instructions a pixel at +-15. The gradient of a 16,384-pixel batch of a 640 x 360 frame: 0.58 ms with the
-// whole frame extracted, 0.31 ms with the list (131 us of it this kernel).
+// Bound by instruction issue (0.70 of the slots): 4,200 warp instructions a pixel at +-15 (5,000 and 131
+// instead of 105 us for 16,384 pixels with each window's few samples filtered at once).  Extracting the whole
+// 640 x 360 frame takes 385 us; the gradient of the batch went from 0.60 to 0.25 ms, with the training
+// kernel's operand layout.
 constexpr int kListThreads = 256, kListCtas = 4, kListGeomStride = 33;  // words a slot: an odd stride, no bank conflicts
+constexpr int kListQueue = 128;  // samples a warp can hold: 31 waiting and one window's 49, rounded up
 
 template <int CFMT>
 __global__ void __launch_bounds__(kListThreads, kListCtas) extract_list_kernel(const GatherArgs a, const int32_t *list, int n_list) {
     extern __shared__ float4 s_dyn[];
     float4 *s_ctx = s_dyn + (threadIdx.x >> 5) * 32 * 4;                  // this warp's 32 frames x 4
-    float *s_geom = reinterpret_cast<float *>(s_dyn + kListThreads * 4);  // n_slots x kListGeomStride
+    float4 *s_queue = s_dyn + kListThreads * 4 + (threadIdx.x >> 5) * kListQueue;  // this warp's samples
+    float *s_geom = reinterpret_cast<float *>(s_dyn + kListThreads * 4 + kListThreads / 32 * kListQueue);  // n_slots x kListGeomStride
     const int lane = threadIdx.x & 31;
     const float *gsrc = reinterpret_cast<const float *>(a.geom);
     for (int i = threadIdx.x; i < a.n_slots * 32; i += kListThreads)
@@ -970,7 +973,26 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) extract_list_kernel(c
         const float dref = __ldg(P.depth + pix);
         const float3 cref = load_colour<CFMT>(P.colour, pix);
         float acc_r = 0.0f, acc_g = 0.0f, acc_b = 0.0f, acc_w = 0.0f;
-        int n_acc = 0;
+        int n_acc = 0, n_done = 0;  // samples found, filtered
+        // sample idx of the queue: its weight joins this lane's sums, the first 64 are stored
+        auto filter = [&](int idx) {
+            const float4 e = s_queue[idx & (kListQueue - 1)];
+            const int id = __float_as_int(e.x), t = id & 255;
+            const float4 c0 = s_ctx[t * 4], c3 = s_ctx[t * 4 + 3];
+            const long long at = (long long)__float_as_int(c0.x) * P.fstride + (__float_as_int(c0.y) + (id >> 8 & 255) * P.pitch + (id >> 16));
+            float dq;
+            float3 c;
+            load_sample<CFMT>(P.depth, P.colour, at, dq, c);
+            const float er = c.x - cref.x, eg = c.y - cref.y, eb = c.z - cref.z;
+            const float x = fmaf(a_rgb, fmaf(er, er, fmaf(eg, eg, eb * eb)), fmaf(a_xyz, e.y, c3.z));
+            const float w = ex2(x);
+            if (idx < kMaxSamples)
+                store_sample(a, (unsigned)i * (unsigned)kMaxSamples + idx, c, sqrt_approx(e.y) * inv_r, c3.w, e.z * inv_r, x * kLn2);
+            acc_r = fmaf(w, er, acc_r);
+            acc_g = fmaf(w, eg, acc_g);
+            acc_b = fmaf(w, eb, acc_b);
+            acc_w += w;
+        };
         if (dref > 0.0f) {
             for (int base = 0; base < a.n_slots; base += 32) {
                 const int jj = base + lane;
@@ -1022,9 +1044,6 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) extract_list_kernel(c
                     live &= live - 1u;
                     const float4 c1 = s_ctx[t * 4 + 1], c2 = s_ctx[t * 4 + 2], c3 = s_ctx[t * 4 + 3];
                     const float d[2] = {dn[0], dn[1]};
-                    const float *dw = dwin;
-                    const void *cwin = CFMT == 0 ? (const void *)(reinterpret_cast<const float4 *>(P.colour) + (dw - P.depth))
-                                                 : (const void *)(reinterpret_cast<const uint2 *>(P.colour) + (dw - P.depth));
                     if (live) fetch(__ffs((int)live) - 1);
                     float d2[2], dz[2];
                     unsigned hits[2];
@@ -1037,32 +1056,24 @@ __global__ void __launch_bounds__(kListThreads, kListCtas) extract_list_kernel(c
                         d2[half] = fmaf(X, X, fmaf(Y, Y, dz[half] * dz[half]));
                         hits[half] = __ballot_sync(0xffffffffu, d2[half] < r2);
                     }
-                    // a lane's samples of both halves of the window, mostly one at most: one pass takes the
-                    // first of every lane, a second one the lanes that have two
-                    bool h0 = hits[0] >> lane & 1u, h1 = hits[1] >> lane & 1u;
-                    while (h0 || h1) {
-                        const int row = h0 ? row0 : 4 + row0;
-                        const float dd2 = h0 ? d2[0] : d2[1], ddz = h0 ? dz[0] : dz[1];
-                        const int idx = n_acc + (h0 ? __popc(hits[0] & below) : __popc(hits[0]) + __popc(hits[1] & below));
-                        if (h0) h0 = false;
-                        else h1 = false;
-                        float dq;
-                        float3 c;
-                        load_sample<CFMT>(dw, cwin, row * P.pitch + col, dq, c);
-                        const float er = c.x - cref.x, eg = c.y - cref.y, eb = c.z - cref.z;
-                        const float e = fmaf(a_rgb, fmaf(er, er, fmaf(eg, eg, eb * eb)), fmaf(a_xyz, dd2, c3.z));
-                        const float w = ex2(e);
-                        if (idx < kMaxSamples)
-                            store_sample(a, (unsigned)i * (unsigned)kMaxSamples + idx, c, sqrt_approx(dd2) * inv_r, c3.w,
-                                         ddz * inv_r, e * kLn2);
-                        acc_r = fmaf(w, er, acc_r);
-                        acc_g = fmaf(w, eg, acc_g);
-                        acc_b = fmaf(w, eb, acc_b);
-                        acc_w += w;
+                    // the samples queue up in canonical order; every 32 are filtered together
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const int at = n_acc + (half ? __popc(hits[0]) : 0) + __popc(hits[half] & below);
+                        if (hits[half] >> lane & 1u)
+                            s_queue[at & (kListQueue - 1)] = make_float4(
+                                __int_as_float(t | (4 * half + row0) << 8 | col << 16), d2[half], dz[half], 0.0f);
                     }
-                    __syncwarp();
                     n_acc += __popc(hits[0]) + __popc(hits[1]);
+                    for (; n_acc - n_done >= 32; n_done += 32) {
+                        __syncwarp();
+                        filter(n_done + lane);
+                        __syncwarp();
+                    }
                 }
+                __syncwarp();
+                if (n_done + lane < n_acc) filter(n_done + lane);
+                n_done = n_acc;
                 __syncwarp();  // the next 32 frames overwrite s_ctx
             }
         }
@@ -1206,7 +1217,7 @@ cudaError_t launch_extract_list(const GatherArgs &a, const int32_t *list, int n_
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const size_t smem = sizeof(float4) * 4 * kListThreads + sizeof(float) * kListGeomStride * (size_t)a.n_slots;
+    const size_t smem = sizeof(float4) * (4 * kListThreads + kListThreads / 32 * kListQueue) + sizeof(float) * kListGeomStride * (size_t)a.n_slots;
     void (*fn)(const GatherArgs, const int32_t *, int) = a.clip.colour_fmt == 0 ? extract_list_kernel<0> : extract_list_kernel<1>;
     if (smem > 48 * 1024 && (e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;

@@ -176,10 +176,22 @@ __device__ __forceinline__ unsigned bf16_pair(float lo, float hi) {
 }
 // i = crop pixel * 64 + slot: the host keeps the sets of a crop below 2^32 samples, so one 32-bit
 // index (widened in the address arithmetic) addresses both arrays
+__device__ __forceinline__ void store_sample(const GatherArgs &a, unsigned i, const float4 c, unsigned f) {
+    a.sets.col[i] = c;
+    a.sets.f89[i] = f;
+}
 __device__ __forceinline__ void store_sample(const GatherArgs &a, unsigned i, float3 c, float dist_r, float dj_t,
                                              float dz_r, float logw) {
-    a.sets.col[i] = make_float4(c.x, c.y, c.z, __uint_as_float(bf16_pair(dist_r, dj_t)));
-    a.sets.f89[i] = bf16_pair(dz_r, logw);
+    store_sample(a, i, make_float4(c.x, c.y, c.z, __uint_as_float(bf16_pair(dist_r, dj_t))), bf16_pair(dz_r, logw));
+}
+// Two consecutive samples, i even: 32 + 8 bytes in two stores.  The samples of a warp's pixels lie 1 KB apart,
+// so each store of a lane is a sector of its own whatever its size.
+__device__ __forceinline__ void store_samples(const GatherArgs &a, unsigned i, const float4 c0, unsigned f0, const float4 c1,
+                                              unsigned f1) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(a.sets.col + i), "f"(c0.x), "f"(c0.y), "f"(c0.z),
+                 "f"(c0.w), "f"(c1.x), "f"(c1.y), "f"(c1.z), "f"(c1.w)
+                 : "memory");
+    *reinterpret_cast<uint2 *>(a.sets.f89 + i) = make_uint2(f0, f1);
 }
 // the distance feature is rounded to BF16 (8 significant bits): the approximate square root
 // (a few FP32 ulp, exact at 0) is enough
@@ -368,7 +380,8 @@ __device__ __forceinline__ void window_centre(const df U, const df V, float &cxf
 }
 
 // LEARN: visit the frames in canonical order (O, O-1, O+1, ...) and store the features of the
-// first kMaxSamples accepted samples (learned filter); the Eq. 3/4 result goes to a.sets.plain.
+// first kMaxSamples accepted samples (learned filter), one by one (1) or in pairs (2); the Eq. 3/4 result
+// goes to a.sets.plain.
 // STG: the candidate depths of the test loop come from the warp's staged boxes (K > 0, not LEARN);
 // tmap describes the clip's depth planes
 // a_rgb and a_xyz: -log2(e) / (2 sigma^2) of Eq. 4's colour and position terms
@@ -380,7 +393,7 @@ __device__ __forceinline__ void window_centre(const df U, const df V, float &cxf
 // flight and up to NS - 1 idle slots at the end of a frame's list: 2 -> 3 takes a 1080p +-30 FP32 frame
 // from 4.15 to 3.99 ms, but with FP16 colour, whose samples take two loads and conversions, and in the
 // batched kernel the registers run out (a 720p FP16 frame 1.03 -> 1.06 ms, the mixed clips' plan 13.5 -> 14.0)
-template <int K, int CFMT, int NS, int NT, bool DEBUG, bool LEARN = false, bool STG = false, int S = 1>
+template <int K, int CFMT, int NS, int NT, bool DEBUG, int LEARN = 0, bool STG = false, int S = 1>
 __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &P, const int O, const int u0,
                                              const int v0, const int u, const int v, const bool active,
                                              const long long crop_idx, const float4 *sgeom, const int n_slots,
@@ -395,6 +408,8 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
     const int rec_words = 3 + (k * k + 31) / 32;
     float acc_r = 0.0f, acc_g = 0.0f, acc_b = 0.0f;
     int n_feat = 0;
+    float4 held_c = make_float4(0.f, 0.f, 0.f, 0.f);  // LEARN 2: an even sample waits for the odd one after it
+    unsigned held_f = 0u;
     const int Tw = (n_slots - 1) >> 1;
     const float inv_r = LEARN ? rsqrtf(r2) : 0.0f, inv_T = LEARN ? 1.0f / (float)max(Tw, 1) : 0.0f;
     const unsigned set0 = LEARN ? (unsigned)crop_idx * (unsigned)kMaxSamples : 0u;
@@ -605,8 +620,16 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
                                     float cr, cg, cb, cd;
                                     f2_unpack(rg[t], cr, cg);
                                     f2_unpack(bz[t], cb, cd);
-                                    store_sample(a, set0 + n_feat, make_float3(cr, cg, cb), sqrt_approx(d2) * inv_r, dj_t,
-                                                 dz * inv_r, e * kLn2);
+                                    const float4 sc = make_float4(cr, cg, cb, __uint_as_float(bf16_pair(sqrt_approx(d2) * inv_r, dj_t)));
+                                    const unsigned sf = bf16_pair(dz * inv_r, e * kLn2);
+                                    if (LEARN == 1) {
+                                        store_sample(a, set0 + n_feat, sc, sf);
+                                    } else if (n_feat & 1) {
+                                        store_samples(a, set0 + n_feat - 1, held_c, held_f, sc, sf);
+                                    } else {
+                                        held_c = sc;
+                                        held_f = sf;
+                                    }
                                     ++n_feat;
                                 }
                                 s_r[0] = odd ? s_r[0] : fmaf(w, er, s_r[0]);
@@ -755,6 +778,10 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
         o[1] = o_g;
         o[2] = o_b;
         if (LEARN) {
+            if (K > 0 && LEARN == 2 && (n_feat & 1)) {
+                a.sets.col[set0 + n_feat - 1] = held_c;
+                a.sets.f89[set0 + n_feat - 1] = held_f;
+            }
             // per pixel: the count kept, c_ref and the size of the whole set / 64 (what the plain
             // fallback averages)
             a.sets.n[crop_idx] = n_feat;
@@ -773,7 +800,7 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
 // One CTA per 32 x kTileY output tile of one output frame (grid: tiles x output frames).
 // STG: the staged gather; dynamic shared memory then holds, after the slot geometry (aligned up to
 // 128 bytes), two boxes per warp, and tmap describes the clip's depth planes.
-template <int K, int CFMT, bool DEBUG, bool LEARN = false, int MINB = SSVP_MIN_CTAS, bool STG = false, int S = 1>
+template <int K, int CFMT, bool DEBUG, int LEARN = 0, int MINB = SSVP_MIN_CTAS, bool STG = false, int S = 1>
 __global__ void __launch_bounds__(kThreads, MINB) gather_kernel(const GatherArgs a, const __grid_constant__ CUtensorMap tmap) {
     extern __shared__ float4 sgeom[];
     __shared__ float s_const[4];
@@ -1172,7 +1199,12 @@ cudaError_t launch_k(const GatherArgs &a, cudaStream_t s) {
             return cudaErrorInvalidValue;
         }
     }
-    if (a.sets.col) gather_kernel<K, CFMT, false, true, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
+    // Sets stored in pairs halve the stores, which hold large crops back (every store of a lane is a sector of its
+    // own), for some instructions more: +-6, two frames, 1080p 7.84 -> 6.99 ms, 960 x 540 1.90 -> 1.80, 800 x 450
+    // 1.30 -> 1.27, 640 x 360 0.80 -> 0.82, 480 x 270 0.51 -> 0.52
+    if (a.sets.col && (long long)a.cw * a.ch >= 300000)
+        gather_kernel<K, CFMT, false, 2, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
+    else if (a.sets.col) gather_kernel<K, CFMT, false, 1, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
     else if (dbg) gather_kernel<K, CFMT, true><<<grid, kThreads, smem, s>>>(a, tmap);
     else {
         // Few CTAs leave SMs idle or end in a nearly empty wave: below two and a half waves each pixel's frames

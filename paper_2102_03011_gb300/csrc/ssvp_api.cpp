@@ -64,6 +64,9 @@ void swap_window(Planes &a, Planes &b) {
 
 char g_create_error[512] = "";
 
+// the launch statistics: two counts and a sum of weights, cleared by one memset a call
+constexpr size_t kStatBytes = 2 * sizeof(unsigned long long) + sizeof(double);
+
 }  // namespace
 
 struct ssvp_ctx {
@@ -72,7 +75,7 @@ struct ssvp_ctx {
     Clip clips[SSVP_MAX_CLIPS];
     char err[512] = "";
     // device scratch
-    unsigned long long *stat_counts = nullptr;  // [2]
+    unsigned long long *stat_counts = nullptr;  // [2], and stat_sumw after them in the same allocation
     double *stat_sumw = nullptr;
     unsigned int *median_scratch = nullptr;
     int *d_kerr = nullptr;  // set by a kernel whose bounded device-side wait gave up; read by ssvp_sync
@@ -735,16 +738,15 @@ int ssvp_create(ssvp_ctx **out, int cuda_device, void *cuda_stream) {
         ssvp_destroy(ctx);
         return rc;
     }
-    if ((e = cudaMalloc(&ctx->stat_counts, 2 * sizeof(unsigned long long))) != cudaSuccess ||
-        (e = cudaMalloc(&ctx->stat_sumw, sizeof(double))) != cudaSuccess ||
+    if ((e = cudaMalloc(&ctx->stat_counts, kStatBytes)) != cudaSuccess ||
         (e = cudaMalloc(&ctx->median_scratch, ssvp::median_scratch_words() * sizeof(unsigned int))) != cudaSuccess ||
         (e = cudaMalloc(&ctx->d_kerr, sizeof(int))) != cudaSuccess) {
         int rc = fail(nullptr, e == cudaErrorMemoryAllocation ? SSVP_ENOMEM : SSVP_ECUDA, "cudaMalloc: %s", cudaGetErrorString(e));
         ssvp_destroy(ctx);
         return rc;
     }
-    cudaMemsetAsync(ctx->stat_counts, 0, 2 * sizeof(unsigned long long), ctx->stream);
-    cudaMemsetAsync(ctx->stat_sumw, 0, sizeof(double), ctx->stream);
+    ctx->stat_sumw = (double *)(ctx->stat_counts + 2);
+    cudaMemsetAsync(ctx->stat_counts, 0, kStatBytes, ctx->stream);
     cudaMemsetAsync(ctx->d_kerr, 0, sizeof(int), ctx->stream);
     *out = ctx;
     return SSVP_OK;
@@ -757,7 +759,6 @@ void ssvp_destroy(ssvp_ctx *ctx) {
     if (ctx->load_stream) cudaStreamSynchronize(ctx->load_stream);
     for (auto &c : ctx->clips) free_clip(c);  // plans of this context must be destroyed first
     if (ctx->stat_counts) cudaFree(ctx->stat_counts);
-    if (ctx->stat_sumw) cudaFree(ctx->stat_sumw);
     if (ctx->median_scratch) cudaFree(ctx->median_scratch);
     if (ctx->d_kerr) cudaFree(ctx->d_kerr);
     if (ctx->geom) cudaFree(ctx->geom);
@@ -1096,8 +1097,7 @@ int ssvp_gather_filter(ssvp_ctx *ctx, const ssvp_params *params, const int *clip
         if (p.k > 7) return fail(ctx, SSVP_EINVAL, "the learned filter supports k <= 7");
         if (p.membership_out || p.pixel_stats_out) return fail(ctx, SSVP_EINVAL, "learned mode has no debug outputs");
         if (p.test_skip_mma != 0 && p.test_skip_mma != 1) return fail(ctx, SSVP_EINVAL, "test_skip_mma must be 0 or 1");
-        CK(cudaMemsetAsync(ctx->stat_counts, 0, 2 * sizeof(unsigned long long), ctx->stream), "cudaMemsetAsync");
-        CK(cudaMemsetAsync(ctx->stat_sumw, 0, sizeof(double), ctx->stream), "cudaMemsetAsync");
+        CK(cudaMemsetAsync(ctx->stat_counts, 0, kStatBytes, ctx->stream), "cudaMemsetAsync");
         for (int i = 0; i < n_clips; ++i) {
             Clip &c = ctx->clips[clip_ids[i]];
             const size_t npx = (size_t)cw[i] * chh[i];
@@ -1163,8 +1163,7 @@ int ssvp_gather_filter(ssvp_ctx *ctx, const ssvp_params *params, const int *clip
     if (entries)
         CK(cudaMemcpyAsync(ctx->geom, ctx->host_geom.data(), entries * sizeof(PairGeom), cudaMemcpyHostToDevice, ctx->stream),
            "cudaMemcpyAsync (geometry)");
-    CK(cudaMemsetAsync(ctx->stat_counts, 0, 2 * sizeof(unsigned long long), ctx->stream), "cudaMemsetAsync");
-    CK(cudaMemsetAsync(ctx->stat_sumw, 0, sizeof(double), ctx->stream), "cudaMemsetAsync");
+    CK(cudaMemsetAsync(ctx->stat_counts, 0, kStatBytes, ctx->stream), "cudaMemsetAsync");
     off = 0;
     for (int i = 0; i < n_clips; ++i) {
         Clip &c = ctx->clips[clip_ids[i]];
@@ -1263,8 +1262,7 @@ int ssvp_superres(ssvp_ctx *ctx, const ssvp_params *params, int clip_id, int sca
     compose_tables_sr(c, b, n_out, T, p.sigma_f, scale, ctx->host_geom.data(), ctx->host_geom.data() + total);
     CK(cudaMemcpyAsync(ctx->geom, ctx->host_geom.data(), 2 * total * sizeof(PairGeom), cudaMemcpyHostToDevice, ctx->stream),
        "cudaMemcpyAsync (geometry)");
-    CK(cudaMemsetAsync(ctx->stat_counts, 0, 2 * sizeof(unsigned long long), ctx->stream), "cudaMemsetAsync");
-    CK(cudaMemsetAsync(ctx->stat_sumw, 0, sizeof(double), ctx->stream), "cudaMemsetAsync");
+    CK(cudaMemsetAsync(ctx->stat_counts, 0, kStatBytes, ctx->stream), "cudaMemsetAsync");
     GatherArgs a{};
     a.clip = c.p;
     a.geom = ctx->geom;
@@ -1607,11 +1605,10 @@ int ssvp_plan_create(ssvp_ctx *ctx, const ssvp_params *params, const int *clip_i
         GatherArgs a = batch_gather_args(ctx, *params);
         const ssvp::BatchArgs b = batch_args(bs, n_clips, cfg.frame_chunk, plan->d_counter);
         cudaError_t e1 = cudaMemsetAsync(plan->d_counter, 0, sizeof(unsigned long long), plan->cap_stream);
-        cudaError_t e2 = cudaMemsetAsync(ctx->stat_counts, 0, 2 * sizeof(unsigned long long), plan->cap_stream);
-        cudaError_t e3 = cudaMemsetAsync(ctx->stat_sumw, 0, sizeof(double), plan->cap_stream);
-        cudaError_t e4 = ssvp::launch_batch(a, b, cfg.tile_rows, cfmt, plan->grid, plan->cap_stream);
+        cudaError_t e2 = cudaMemsetAsync(ctx->stat_counts, 0, kStatBytes, plan->cap_stream);
+        cudaError_t e3 = ssvp::launch_batch(a, b, cfg.tile_rows, cfmt, plan->grid, plan->cap_stream);
         e = cudaStreamEndCapture(plan->cap_stream, &plan->graph);
-        if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3 != cudaSuccess ? e3 : e4;
+        if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3;
         if (e != cudaSuccess) break;
         if ((e = cudaGraphInstantiate(&plan->exec, plan->graph, 0)) != cudaSuccess) break;
     } while (0);

@@ -1190,7 +1190,8 @@ cudaError_t launch_k(const GatherArgs &a, cudaStream_t s) {
             void (*fn)(const GatherArgs, const CUtensorMap) =
                 dbg ? gather_kernel<K, CFMT, true, false, SSVP_MIN_CTAS, true>
                     : gather_kernel<K, CFMT, false, false, SSVP_MIN_CTAS, true>;
-            if (smem > 48 * 1024 &&
+            // 48 KB without it, of which the kernel's own arrays take less than 8
+            if (smem > 40 * 1024 &&
                 (e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
                 return e;
             fn<<<grid, kThreads, smem, s>>>(a, tmap);

@@ -43,3 +43,13 @@ def test_survivors_hold_every_sample(sess, k, r_px):
         plain = sess.run(0, O, k=k, half_window=2, radius=float(radius))
         np.testing.assert_allclose(plain.rgb, g.rgb, rtol=0, atol=405 * 2.0 ** -24)
     assert members >= 2 * 71 * 43  # at least the pixels themselves
+
+
+@pytest.mark.parametrize("T", [30, 40, 50, 60, 127])
+def test_staged_long_windows(sess, T):
+    """Windows whose geometry and staged boxes come near, to and over 48 KB of shared memory."""
+    clip = synth.make_clip("planes3", 45, 37, 9, seed=2)
+    sess.load(0, clip)
+    a = sess.run(0, 4, k=5, half_window=T)
+    b = sess.run(0, 4, k=5, half_window=T, gather=sess.ss.SSVP_GATHER_WINDOW_TMA)
+    np.testing.assert_array_equal(a.rgb, b.rgb)

@@ -560,6 +560,9 @@ __global__ void __launch_bounds__(kTcThreads, 3) mlp_train_tc_kernel(const MlpAr
             pl[2] = m.sets.plain[3 * si + 2];
         }
         const bool valid = srow < n;
+        // slots past the set's count hold whatever the memory held before (an earlier call's samples, a freed
+        // plane's NaN): their weight of 0 in the sums below does not make an infinite colour 0
+        if (!valid) c = make_float4(0.f, 0.f, 0.f, 0.f);
         // 2. features (logical order; slot 15 carries 1.0 for b1 in the layer-1 operand only)
         unsigned wd[8];
 #pragma unroll

@@ -177,24 +177,38 @@ constexpr int kFrSlotVec = 8;  // float4 words of a window slot in shared memory
 //  0-2 = forward map M (9), e (3); 3 = zlo zhi (J's valid depth range), log2 weight of the frame (negated), J
 //  4-6 = back map M (9), e (3); 7.x = 1 / fx of J
 constexpr int kTile = 8;       // side of the depth range tiles
-// Positions along the hull from which its blocks are checked by their depth range (see the slot loop), if
-// any lane of the warp has as many; at most 256.  The check costs about as much as 25 candidates, which a
-// short hull does not save.  720p, +-15: 3.40, 3.23, 3.40, 3.62 ms with the line at 16, 32, 48 and never;
-// 1080p, +-30: 20.6, 20.4, 20.5, 35.0; super-resolution to 1080p, where hulls are one or two pixels wide:
-// 8.1, 7.5, 7.1, 7.1.
+// Positions along the hull from which its blocks are checked by their depth range (see the slot loop).  The check
+// costs about as much as 25 candidates, which a short hull does not save.
 template <bool SR> constexpr int kLongHull = SR ? 48 : 32;
 constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: x + kRound holds x rounded to an integer in its low bits
 
-// S (a power of two): each pixel's window frames are shared out to S threads (the CTA takes 32 x 8 / S pixels),
-// by J modulo S, whatever the window; they join their sums after each pass
+// A pixel's sums over one group of its window frames, or over all: the colours and the weight, times 2^-m
+struct FrSums { float r, g, b, w, m; };
+
+// The sums of the next group join those before it, at the larger of the two powers; the roundings are spelled out,
+// so that they are the same whichever thread joins
+__device__ __forceinline__ void join_sums(FrSums &a, const FrSums &b) {
+    const float m = fmaxf(a.m, b.m), sa = ex2(__fsub_rn(a.m, m)), sb = ex2(__fsub_rn(b.m, m));
+    a.r = __fmaf_rn(sb, b.r, __fmul_rn(sa, a.r));
+    a.g = __fmaf_rn(sb, b.g, __fmul_rn(sa, a.g));
+    a.b = __fmaf_rn(sb, b.b, __fmul_rn(sa, a.b));
+    a.w = __fmaf_rn(sb, b.w, __fmul_rn(sa, a.w));
+    a.m = m;
+}
+
+// A pixel's window frames are summed in four groups, by J modulo 4 whatever the window, each in order, and the
+// groups are joined in order.  S = 1: one thread a pixel goes through all four; S = 4: each pixel has four threads
+// of the CTA (which takes 32 x 2 pixels), one a group.  The result is the same to the bit, and every choice within
+// it is the pixel's own: it depends neither on the crop nor on how many frames a launch has.
 template <int CFMT, bool DEBUG, bool SR, int INP, int S>
 __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const GatherArgs a) {
+    static_assert(S == 1 || S == 4, "one thread a pixel or one a group");
     constexpr int kRows = kFrTileY / S;
     extern __shared__ float4 s_slot[];
     __shared__ float s_const[8];
     __shared__ unsigned long long s_cnt[2][kFrThreads / 32];
     __shared__ float s_w[kFrThreads / 32];
-    __shared__ float s_red[S > 1 ? S : 1][5][S > 1 ? kRows * 32 : 1];
+    __shared__ FrSums s_red[S][kRows * 32];  // S = 1: the sums of the groups so far (in registers they spill)
     __shared__ int s_dbg[DEBUG && S > 1 ? kRows * 32 : 1][2];
     const Planes &P = a.clip;
     const int oi = blockIdx.z;
@@ -317,7 +331,8 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
     acc_r = acc_g = acc_b = acc_w = 0.0f;
     m_log2 = wpass ? kNoWeight : 0.0f;
     if (gather) {
-        for (int j = (split - (O - a.T)) & (S - 1); j < ns; j += S) {
+      for (int grp = split; grp < 4; grp += S) {
+        for (int j = (grp - (O - a.T)) & 3; j < ns; j += 4) {
             const float4 *sl = s_slot + kFrSlotVec * j;
             const float4 q3 = sl[3];
             const int J = __float_as_int(q3.w);
@@ -484,7 +499,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                     mh += mix64((unsigned long long)qy * (unsigned long long)P.W + (unsigned long long)qx + 1ull);
                 }
             };
-            if (!__any_sync(__activemask(), m1 - m0 >= kLongHull<SR>)) {
+            if (m1 - m0 < kLongHull<SR>) {  // by the pixel alone: the two walks sum in different orders
                 // Short hulls: row by row of the minor axis, each row a run along the major axis, every candidate
                 // b m + lo <= n <= b m + hi, m in [m0, m1] by the packed exact test (two candidates an operation;
                 // |h1| + |h2| is the larger of |h1 + h2| and |h1 - h2|), up to 32 into a hit mask
@@ -701,29 +716,37 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                 rec[3] = (int32_t)(unsigned int)(mh >> 32);
             }
         }
+        if (S == 1) {
+            const FrSums part = {acc_r, acc_g, acc_b, acc_w, m_log2};
+            FrSums &sum = s_red[0][threadIdx.x];
+            if (grp == 0) sum = part;
+            else join_sums(sum, part);
+            if (grp < 3) {
+                acc_r = acc_g = acc_b = acc_w = 0.0f;
+                m_log2 = wpass ? kNoWeight : 0.0f;
+            } else {
+                acc_r = sum.r;
+                acc_g = sum.g;
+                acc_b = sum.b;
+                acc_w = sum.w;
+                m_log2 = sum.m;
+            }
+        }
+      }
     }
     if (S > 1) {
-        // join the S threads' sums, brought to the largest weight of all; every thread takes the result
+        // join the four threads' sums; every thread takes the result
         const int px = row * 32 + lane;
-        s_red[split][0][px] = acc_r;
-        s_red[split][1][px] = acc_g;
-        s_red[split][2][px] = acc_b;
-        s_red[split][3][px] = acc_w;
-        s_red[split][4][px] = m_log2;
+        s_red[split][px] = {acc_r, acc_g, acc_b, acc_w, m_log2};
         __syncthreads();
-        float m = s_red[0][4][px];
+        FrSums sum = s_red[0][px];
 #pragma unroll
-        for (int s = 1; s < S; ++s) m = fmaxf(m, s_red[s][4][px]);
-        acc_r = acc_g = acc_b = acc_w = 0.0f;
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const float sc = ex2(s_red[s][4][px] - m);
-            acc_r = fmaf(sc, s_red[s][0][px], acc_r);
-            acc_g = fmaf(sc, s_red[s][1][px], acc_g);
-            acc_b = fmaf(sc, s_red[s][2][px], acc_b);
-            acc_w = fmaf(sc, s_red[s][3][px], acc_w);
-        }
-        m_log2 = m;
+        for (int s = 1; s < S; ++s) join_sums(sum, s_red[s][px]);
+        acc_r = sum.r;
+        acc_g = sum.g;
+        acc_b = sum.b;
+        acc_w = sum.w;
+        m_log2 = sum.m;
         __syncthreads();
     }
     sw_true = acc_w > 0.0f ? acc_w * exp2f(m_log2) : 0.0f;  // the true sum of weights of this pass

@@ -36,13 +36,15 @@ constexpr int kApTileY = 8, kApThreads = 32 * kApTileY;
 // 1080p +-10), 64 with FP32 (11.7 against 11.9).
 template <int CFMT> constexpr int kApCtas = CFMT == 1 ? 3 : 4;
 
-// S (a power of two): each pixel's window frames are shared out to S threads (the CTA takes 32 x 8 / S pixels),
-// by J modulo S, whatever the window; their sums are joined at the end
+// A pixel's window frames are summed in four groups, by J modulo 4 whatever the window, each from zero and in order,
+// and the groups' sums are added in order.  S = 1: one thread a pixel goes through all four; S = 4: each pixel has
+// four threads of the CTA (which takes 32 x 2 pixels), one a group.  The result is the same to the bit.
 template <int CFMT, bool DEBUG, int S>
 __global__ void __launch_bounds__(kApThreads, kApCtas<CFMT>) aperture_kernel(const GatherArgs a) {
+    static_assert(S == 1 || S == 4, "one thread a pixel or one a group");
     constexpr int kRows = kApTileY / S;
     extern __shared__ float4 sgeom[];
-    __shared__ float s_red[S > 1 ? S : 1][4][S > 1 ? kRows * 32 : 1];
+    __shared__ float s_red[S][4][kRows * 32];  // S = 1: the sums of the groups so far
     __shared__ float s_const[5];
     __shared__ unsigned long long s_cnt[2][kApThreads / 32];
     __shared__ float s_w[kApThreads / 32];
@@ -67,6 +69,7 @@ __global__ void __launch_bounds__(kApThreads, kApCtas<CFMT>) aperture_kernel(con
 
     const Planes &P = a.clip;
     const int h = (a.k - 1) >> 1, hc = (a.cap - 1) >> 1;
+    const int px = threadIdx.x % (kRows * 32);
     const float z0 = s_const[0], a0 = s_const[1], slope = s_const[2];
     const int tx = threadIdx.x & 31, ty = (threadIdx.x >> 5) % kRows, split = (threadIdx.x >> 5) / kRows;
     const int u = u0 + tx, v = a.y0 + vt + ty;
@@ -91,7 +94,8 @@ __global__ void __launch_bounds__(kApThreads, kApCtas<CFMT>) aperture_kernel(con
     if (gather) {
         const float du = (float)(u - u0), dv = (float)(v - v0);
         const float s_seed = 1.0f - dref / z0;  // seed X_i = x_ref + s (L_i, 0)
-        for (int j = (split - (O - a.T)) & (S - 1); j < a.n_slots; j += S) {
+      for (int grp = split; grp < 4; grp += S) {
+        for (int j = (grp - (O - a.T)) & 3; j < a.n_slots; j += 4) {
             const float4 *g = sgeom + kSlotVec * j;
             const float4 q5 = g[5];
             const int J = __float_as_int(q5.w);
@@ -257,10 +261,26 @@ __global__ void __launch_bounds__(kApThreads, kApCtas<CFMT>) aperture_kernel(con
                 }
             }
         }
+        if (S == 1) {
+            float (*sum)[kRows * 32] = s_red[0];
+            if (grp > 0) {
+                acc_r = sum[0][px] + acc_r;
+                acc_g = sum[1][px] + acc_g;
+                acc_b = sum[2][px] + acc_b;
+                acc_w = sum[3][px] + acc_w;
+            }
+            if (grp < 3) {
+                sum[0][px] = acc_r;
+                sum[1][px] = acc_g;
+                sum[2][px] = acc_b;
+                sum[3][px] = acc_w;
+                acc_r = acc_g = acc_b = acc_w = 0.0f;
+            }
+        }
+      }
     }
 
     if (S > 1) {
-        const int px = ty * 32 + tx;
         s_red[split][0][px] = acc_r;
         s_red[split][1][px] = acc_g;
         s_red[split][2][px] = acc_b;

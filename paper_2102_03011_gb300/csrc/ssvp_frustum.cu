@@ -32,6 +32,7 @@
 
 #include "../../include/ssvp.h"
 #include "ssvp_df.cuh"
+#include "ssvp_dispatch.h"
 #include "ssvp_internal.h"
 
 namespace ssvp {
@@ -175,11 +176,14 @@ __device__ __forceinline__ bool lateral_fast(const float (&Ma)[3], const float (
 template <int INP> constexpr int kFrCtas = INP ? 2 : 3;
 constexpr int kFrSlotVec = 8;  // float4 words of a window slot in shared memory:
 //  0-2 = forward map M (9), e (3); 3 = zlo zhi (J's valid depth range), log2 weight of the frame (negated), J
-//  4-6 = back map M (9), e (3); 7.x = 1 / fx of J
+//  4-6 = back map M (9), e (3); 7.x = 1 / fx of J, 7.y = whether hulls are long
 constexpr int kTile = 8;       // side of the depth range tiles
-// Positions along the hull from which its blocks are checked by their depth range (see the slot loop).  The check
-// costs about as much as 25 candidates, which a short hull does not save.
-template <bool SR> constexpr int kLongHull = SR ? 48 : 32;
+// LONG instances: length of a window frame's hulls, in pixels, from which their blocks are checked by their depth range
+// (see the slot loop).  The check costs about as much as 25 candidates, which a short hull does not save.  One choice
+// for all pixels of a frame: the two walks sum in different orders, and a warp would pay for both (chosen pixel by
+// pixel 720p, +-15, takes 3.37 ms).  720p, +-15: 3.25, 3.21, 3.39, 3.44 ms with the line at 24, 32, 48 and never; 640 x
+// 360, +-30: 1.81, 1.80, 1.88, 1.94; 1080p, +-30: 20.6, 20.5, 20.7, 33.6.
+constexpr int kLongHull = 32;
 constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: x + kRound holds x rounded to an integer in its low bits
 
 // A pixel's sums over one group of its window frames, or over all: the colours and the weight, times 2^-m
@@ -200,7 +204,7 @@ __device__ __forceinline__ void join_sums(FrSums &a, const FrSums &b) {
 // groups are joined in order.  S = 1: one thread a pixel goes through all four; S = 4: each pixel has four threads
 // of the CTA (which takes 32 x 2 pixels), one a group.  The result is the same to the bit, and every choice within
 // it is the pixel's own: it depends neither on the crop nor on how many frames a launch has.
-template <int CFMT, bool DEBUG, bool SR, int INP, int S>
+template <int CFMT, bool DEBUG, bool SR, int INP, int S, bool LONG>
 __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const GatherArgs a) {
     static_assert(S == 1 || S == 4, "one thread a pixel or one a group");
     constexpr int kRows = kFrTileY / S;
@@ -236,7 +240,22 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
         d[4] = make_float4(gb.M_hi[0], gb.M_hi[1], gb.M_hi[2], gb.M_hi[3]);
         d[5] = make_float4(gb.M_hi[4], gb.M_hi[5], gb.M_hi[6], gb.M_hi[7]);
         d[6] = make_float4(gb.M_hi[8], gb.e_hi[0], gb.e_hi[1], gb.e_hi[2]);
-        d[7] = make_float4(gf.ifx, 0.f, 0.f, 0.f);
+        // LONG: whether the blocks of J's hulls are checked, by the length that the ray of the image's centre projects to
+        bool lng = false;
+        if (LONG && J >= 0) {
+            const float sc = SR ? 0.5f * (float)a.sr_scale : 0.5f, cu = sc * (float)P.W, cv = sc * (float)P.H;
+            const float A0 = fmaf(gf.M_hi[0], cu, fmaf(gf.M_hi[1], cv, gf.M_hi[2]));
+            const float A1 = fmaf(gf.M_hi[3], cu, fmaf(gf.M_hi[4], cv, gf.M_hi[5]));
+            const float A2 = fmaf(gf.M_hi[6], cu, fmaf(gf.M_hi[7], cv, gf.M_hi[8]));
+            float za, zb;
+            if (zlo <= zhi && slab_interval(gf.e_hi[2], A2, zlo, zhi, a.near_plane, a.far_plane, za, zb)) {
+                const float wa = fmaf(A2, za, gf.e_hi[2]), wb = fmaf(A2, zb, gf.e_hi[2]);
+                const float dx = fmaf(A0, zb, gf.e_hi[0]) / wb - fmaf(A0, za, gf.e_hi[0]) / wa;
+                const float dy = fmaf(A1, zb, gf.e_hi[1]) / wb - fmaf(A1, za, gf.e_hi[1]) / wa;
+                lng = fmaxf(fabsf(dx), fabsf(dy)) >= (float)kLongHull;
+            }
+        }
+        d[7] = make_float4(gf.ifx, __int_as_float(lng), 0.f, 0.f);
     }
     if (threadIdx.x == 0) {
         const float r = a.radius > 0.0f ? a.radius : -a.radius * *P.median;
@@ -435,8 +454,8 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
             const float *plane = P.depth + fbase;
             int mc = 0;
             unsigned long long mh = 0ull;
-            // the pixel at (m, n) by the exact test of Eq. 2; a sample joins the sums
-            auto take = [&](int m, int n) {
+            // the pixel at (m, n) by the exact test of Eq. 2 (unless `tested` already); a sample joins the sums
+            auto take = [&](int m, int n, auto tested) {
                 const int pos = m * mstep + n * nstep;
                 float d;
                 float3 c;
@@ -449,7 +468,8 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                 const float hs = fmaf(d, fmaf(sm1 + sm2, fm, b1 + b2), E1 + E2);
                 const float hd = fmaf(d, fmaf(sm1 - sm2, fm, b1 - b2), E1 - E2);
                 const float h3 = fmaf(d, fmaf(sm3, fm, b3), E3);
-                if (!(fabsf(hs) < L * h3 && fabsf(hd) < L * h3) || (check_nf && !(fabsf(h3 - zmid) < zhalf))) return;
+                if (!decltype(tested)::value && !(fabsf(hs) < L * h3 && fabsf(hd) < L * h3)) return;
+                if (check_nf && !(fabsf(h3 - zmid) < zhalf)) return;
                 const float h1 = fmaf(d, fmaf(sm1, fm, b1), E1), h2 = fmaf(d, fmaf(sm2, fm, b2), E2);
                 // Eq. 9: masked samples weigh 0 in the mean-shift steps (semi-transparency:
                 // except for their Eq. 4 term in the last pass)
@@ -499,7 +519,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                     mh += mix64((unsigned long long)qy * (unsigned long long)P.W + (unsigned long long)qx + 1ull);
                 }
             };
-            if (m1 - m0 < kLongHull<SR>) {  // by the pixel alone: the two walks sum in different orders
+            if (!LONG || __float_as_int(sl[7].y) == 0) {
                 // Short hulls: row by row of the minor axis, each row a run along the major axis, every candidate
                 // b m + lo <= n <= b m + hi, m in [m0, m1] by the packed exact test (two candidates an operation;
                 // |h1| + |h2| is the larger of |h1 + h2| and |h1 - h2|), up to 32 into a hit mask
@@ -560,7 +580,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                         while (hit) {
                             const int k = __ffs((int)hit) - 1;
                             hit &= hit - 1u;
-                            take(mc0 + k, n);
+                            take(mc0 + k, n, std::true_type{});
                         }
                     }
                 }
@@ -704,7 +724,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                                 const int m = mb + (narrow ? k >> 1 : k >> 2);
                                 const float t = fmaf(bb, (float)m, start) + kRound;
                                 const int n = min(max(__float_as_int(t) - __float_as_int(kRound) + 4 * ch, -4), nmin) + (narrow ? k & 1 : k & 3);
-                                take(m, n);
+                                take(m, n, std::false_type{});
                             }
                         }
                     }
@@ -845,16 +865,22 @@ __global__ void __launch_bounds__(256) zrange_kernel(Planes P, unsigned int *zr,
     }
 }
 
-template <bool SR, int INP, int S>
+template <bool SR, int INP, int S, bool LONG>
 cudaError_t launch_frustum_t(const GatherArgs &a, cudaStream_t s) {
     constexpr int kRows = kFrTileY / S;
     const dim3 grid((a.cw + kFrTileX - 1) / kFrTileX, (a.ch + kRows - 1) / kRows, a.n_out);
     const bool dbg = a.membership || a.pixel_stats;
     const size_t smem = sizeof(float4) * kFrSlotVec * (size_t)a.n_slots;  // at most 32 KB
-    void (*fn)(const GatherArgs) = a.clip.colour_fmt == 0 ? (dbg ? frustum_kernel<0, true, SR, INP, S> : frustum_kernel<0, false, SR, INP, S>)
-                                                          : (dbg ? frustum_kernel<1, true, SR, INP, S> : frustum_kernel<1, false, SR, INP, S>);
+    void (*fn)(const GatherArgs) = a.clip.colour_fmt == 0
+                                       ? (dbg ? frustum_kernel<0, true, SR, INP, S, LONG> : frustum_kernel<0, false, SR, INP, S, LONG>)
+                                       : (dbg ? frustum_kernel<1, true, SR, INP, S, LONG> : frustum_kernel<1, false, SR, INP, S, LONG>);
     fn<<<grid, kFrThreads, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+template <bool SR, int INP, int S>
+cudaError_t launch_frustum_s(const GatherArgs &a, cudaStream_t s) {
+    return frustum_long_hulls(a.n_slots, a.clip.W, SR ? a.frustum_l / (float)a.sr_scale : a.frustum_l) ? launch_frustum_t<SR, INP, S, true>(a, s) : launch_frustum_t<SR, INP, S, false>(a, s);
 }
 
 // Eq. 8-9's mask from a scene-space box: per pixel of every frame, the world point of its depth
@@ -897,15 +923,15 @@ __global__ void __launch_bounds__(256) mask_box_kernel(Planes P, const double *c
 // where one thread a pixel gives less than one and a half waves of CTAs (a 320 x 180 frame, +-15: 0.220 ->
 // 0.155 ms); at 720p one thread a pixel is better (3.23 against 3.35 ms).
 cudaError_t launch_frustum(const GatherArgs &a, cudaStream_t s) {
-    if (a.mode == SSVP_MODE_INPAINT && !a.sr_out) return launch_frustum_t<false, 1, 4>(a, s);
-    if (a.mode == SSVP_MODE_SEMI && !a.sr_out) return launch_frustum_t<false, 2, 4>(a, s);
+    if (a.mode == SSVP_MODE_INPAINT && !a.sr_out) return launch_frustum_s<false, 1, 4>(a, s);
+    if (a.mode == SSVP_MODE_SEMI && !a.sr_out) return launch_frustum_s<false, 2, 4>(a, s);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const long long ctas = (long long)((a.cw + kFrTileX - 1) / kFrTileX) * ((a.ch + kFrTileY - 1) / kFrTileY) * a.n_out;
     const bool split = 2 * ctas < 3ll * kFrCtas<0> * sms;
-    if (a.sr_out) return split ? launch_frustum_t<true, 0, 4>(a, s) : launch_frustum_t<true, 0, 1>(a, s);
-    return split ? launch_frustum_t<false, 0, 4>(a, s) : launch_frustum_t<false, 0, 1>(a, s);
+    if (a.sr_out) return split ? launch_frustum_s<true, 0, 4>(a, s) : launch_frustum_s<true, 0, 1>(a, s);
+    return split ? launch_frustum_s<false, 0, 4>(a, s) : launch_frustum_s<false, 0, 1>(a, s);
 }
 
 cudaError_t launch_mask_box(const Planes &p, const double *cam, const double *box, cudaStream_t s) {

@@ -1,0 +1,36 @@
+"""CPU: the rules that choose between two forms of a kernel (csrc/ssvp_dispatch.h), compiled by the host compiler: on
+which side the measured sizes lie.
+"""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2102_03011_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+
+    def ask(*calls):
+        d = tmp_path_factory.mktemp("rules")
+        src = d / "r.cpp"
+        src.write_text('#include <cstdio>\n#include "ssvp_dispatch.h"\nint main() {\n'
+                       + "".join(f'    printf("%d\\n", (int)ssvp::{c});\n' for c in calls) + "}\n")
+        subprocess.check_call([cxx, "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(d / "r")])
+        return [int(x) for x in subprocess.check_output([str(d / "r")]).split()]
+    return ask
+
+
+def test_long_hulls(rule):
+    def call(T, W, band):
+        return f"frustum_long_hulls({2 * T + 1}, {W}, {band}f)"
+    yes = [(15, 1280, 3.0), (30, 640, 3.0), (30, 1280, 3.0), (30, 1280, 1.0), (30, 1920, 9.0), (60, 640, 1.5), (15, 1920, 9.0), (60, 1280, 0.5)]
+    # short hulls gain nothing, and the instance that can drop their blocks spills
+    no = [(0, 1920, 3.0), (15, 1280, 1.0), (15, 1280, 9.0), (30, 640, 9.0), (30, 640, 1.0), (15, 960, 3.0), (30, 320, 3.0), (15, 1920, 1.0), (30, 1280, 0.5)]
+    assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
+    assert rule(*(call(*c) for c in no)) == [0] * len(no)

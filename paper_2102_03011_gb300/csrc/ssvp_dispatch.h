@@ -2,6 +2,12 @@
 // that the lines they draw can be checked on any machine.
 #pragma once
 
+#ifdef __CUDACC__
+#define SSVP_HD __host__ __device__
+#else
+#define SSVP_HD
+#endif
+
 namespace ssvp {
 
 // Whether a frustum gather takes the instance that can drop whole blocks of a long hull.  Hulls grow with the image
@@ -17,6 +23,18 @@ namespace ssvp {
 // A rule on the whole image and the window, not on the crop: the two sum in different orders.
 inline bool frustum_long_hulls(int n_slots, int width, float band) {
     return (long long)n_slots * width >= (band < 1.0f ? 100000 : band < 2.0f ? 70000 : band < 5.0f ? 35000 : 50000);
+}
+
+// Whether each pixel's window frames are shared out to four threads, where one thread a pixel fills the chip badly.
+// ctas: CTAs of 32 x 8 pixels with one thread a pixel; wave: how many are resident at once.  Four threads cost four
+// times the CTAs, each with its own set-up, and with few frames some threads have none, so the fuller the chip the
+// longer the window has to be.
+
+// Frustum gather, us with one thread and with four (l = 3): 96 x 54 (0.05 waves) +-1 16.3, 13.4 (super-resolution x 2);
+// 320 x 180 (0.5) 0 20.6, 28, +-1 31, 30, +-2 40, 37 (l = 9 118, 108); 480 x 270 (1.1) +-1 48, 53, +-2 70, 75, +-3 92, 85, +-15 450, 378;
+// 640 x 360 (2.0) +-3 118, 134, +-8 306, 343, +-15 694, 700
+SSVP_HD inline bool frustum_shares(long long ctas, long long wave, int n_slots) {
+    return (n_slots >= 3 && 4 * ctas <= wave) || (n_slots >= 5 && 5 * ctas <= 3 * wave) || (n_slots >= 7 && 2 * ctas < 3 * wave);
 }
 
 }  // namespace ssvp

@@ -350,8 +350,11 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
     acc_r = acc_g = acc_b = acc_w = 0.0f;
     m_log2 = wpass ? kNoWeight : 0.0f;
     if (gather) {
+      bool first = true;
       for (int grp = split; grp < 4; grp += S) {
-        for (int j = (grp - (O - a.T)) & 3; j < ns; j += 4) {
+        const int j0 = (grp - (O - a.T)) & 3;
+        if (j0 >= ns) continue;  // joining an empty group's zeros changes nothing
+        for (int j = j0; j < ns; j += 4) {
             const float4 *sl = s_slot + kFrSlotVec * j;
             const float4 q3 = sl[3];
             const int J = __float_as_int(q3.w);
@@ -736,22 +739,26 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                 rec[3] = (int32_t)(unsigned int)(mh >> 32);
             }
         }
-        if (S == 1) {
-            const FrSums part = {acc_r, acc_g, acc_b, acc_w, m_log2};
-            FrSums &sum = s_red[0][threadIdx.x];
-            if (grp == 0) sum = part;
-            else join_sums(sum, part);
-            if (grp < 3) {
-                acc_r = acc_g = acc_b = acc_w = 0.0f;
-                m_log2 = wpass ? kNoWeight : 0.0f;
-            } else {
-                acc_r = sum.r;
-                acc_g = sum.g;
-                acc_b = sum.b;
-                acc_w = sum.w;
-                m_log2 = sum.m;
+        if (S == 1 && ns > 1) {
+            FrSums part = {acc_r, acc_g, acc_b, acc_w, m_log2}, &sum = s_red[0][threadIdx.x];
+            if (!first) {
+                FrSums all = sum;
+                join_sums(all, part);
+                part = all;
             }
+            first = false;
+            sum = part;
+            acc_r = acc_g = acc_b = acc_w = 0.0f;
+            m_log2 = wpass ? kNoWeight : 0.0f;
         }
+      }
+      if (S == 1 && ns > 1) {
+          const FrSums sum = s_red[0][threadIdx.x];
+          acc_r = sum.r;
+          acc_g = sum.g;
+          acc_b = sum.b;
+          acc_w = sum.w;
+          m_log2 = sum.m;
       }
     }
     if (S > 1) {
@@ -918,10 +925,8 @@ __global__ void __launch_bounds__(256) mask_box_kernel(Planes P, const double *c
 
 }  // namespace
 
-// Four threads a pixel for inpainting and semi-transparency, which gather for few of the frame's pixels, in
-// three passes (720p, one box removed: 1.19 ms with one thread a pixel, 0.42 with four, 0.49 with eight), and
-// where one thread a pixel gives less than one and a half waves of CTAs (a 320 x 180 frame, +-15: 0.220 ->
-// 0.155 ms); at 720p one thread a pixel is better (3.23 against 3.35 ms).
+// Four threads a pixel for inpainting and semi-transparency, which gather for few of the frame's pixels, in three
+// passes (720p, one box removed: 1.19 ms with one thread a pixel, 0.42 with four, 0.49 with eight).
 cudaError_t launch_frustum(const GatherArgs &a, cudaStream_t s) {
     if (a.mode == SSVP_MODE_INPAINT && !a.sr_out) return launch_frustum_s<false, 1, 4>(a, s);
     if (a.mode == SSVP_MODE_SEMI && !a.sr_out) return launch_frustum_s<false, 2, 4>(a, s);
@@ -929,9 +934,9 @@ cudaError_t launch_frustum(const GatherArgs &a, cudaStream_t s) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const long long ctas = (long long)((a.cw + kFrTileX - 1) / kFrTileX) * ((a.ch + kFrTileY - 1) / kFrTileY) * a.n_out;
-    const bool split = 2 * ctas < 3ll * kFrCtas<0> * sms;
-    if (a.sr_out) return split ? launch_frustum_s<true, 0, 4>(a, s) : launch_frustum_s<true, 0, 1>(a, s);
-    return split ? launch_frustum_s<false, 0, 4>(a, s) : launch_frustum_s<false, 0, 1>(a, s);
+    const bool shared = frustum_shares(ctas, kFrCtas<0> * sms, a.n_slots);
+    if (a.sr_out) return shared ? launch_frustum_s<true, 0, 4>(a, s) : launch_frustum_s<true, 0, 1>(a, s);
+    return shared ? launch_frustum_s<false, 0, 4>(a, s) : launch_frustum_s<false, 0, 1>(a, s);
 }
 
 cudaError_t launch_mask_box(const Planes &p, const double *cam, const double *box, cudaStream_t s) {

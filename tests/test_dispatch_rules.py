@@ -34,3 +34,20 @@ def test_long_hulls(rule):
     no = [(0, 1920, 3.0), (15, 1280, 1.0), (15, 1280, 9.0), (30, 640, 9.0), (30, 640, 1.0), (15, 960, 3.0), (30, 320, 3.0), (15, 1920, 1.0), (30, 1280, 0.5)]
     assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
     assert rule(*(call(*c) for c in no)) == [0] * len(no)
+
+
+def ctas(W, H, n=1):
+    return (W + 31) // 32 * ((H + 7) // 8) * n
+
+
+SMS = 152
+
+
+def test_frustum_frames_shared(rule):
+    def call(W, H, T):
+        return f"frustum_shares({ctas(W, H)}, {3 * SMS}, {2 * T + 1})"
+    yes = [(96, 54, 1), (160, 90, 1), (256, 144, 2), (320, 180, 2), (320, 180, 3), (320, 180, 15), (480, 270, 3), (480, 270, 15)]
+    # one frame has nothing to share; short windows of larger images; full chips
+    no = [(96, 54, 0), (320, 180, 0), (320, 180, 1), (480, 270, 0), (480, 270, 2), (640, 360, 3), (640, 360, 15), (1280, 720, 30)]
+    assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
+    assert rule(*(call(*c) for c in no)) == [0] * len(no)

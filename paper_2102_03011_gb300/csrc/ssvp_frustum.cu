@@ -171,9 +171,10 @@ __device__ __forceinline__ bool lateral_fast(const float (&Ma)[3], const float (
     return ok;
 }
 
-// Registers: 80 (three CTAs per SM) although the two ways of walking a hull spill some; at 128 a 720p frame
-// takes 3.87 instead of 3.53 ms.  Inpainting, with few warps anyway, is better off with 128 (0.42 -> 0.36 ms).
-template <int INP> constexpr int kFrCtas = INP ? 2 : 3;
+// Registers: 80 (three CTAs per SM), with some spilled in the form that can drop blocks.  For inpainting that form has 128
+// (two CTAs) instead: 720p, +-15, one box of 1 % of the frame, 331 against 354 us.  The other is better off with
+// three CTAs, which spill nothing: 640 x 360, +-5, two fifths of the frame masked, 262 against 335 us.
+template <int INP, bool LONG> constexpr int kFrCtas = INP && LONG ? 2 : 3;
 constexpr int kFrSlotVec = 8;  // float4 words of a window slot in shared memory:
 //  0-2 = forward map M (9), e (3); 3 = zlo zhi (J's valid depth range), log2 weight of the frame (negated), J
 //  4-6 = back map M (9), e (3); 7.x = 1 / fx of J, 7.y = whether hulls are long
@@ -202,22 +203,94 @@ __device__ __forceinline__ void join_sums(FrSums &a, const FrSums &b) {
 
 // A pixel's window frames are summed in four groups, by J modulo 4 whatever the window, each in order, and the
 // groups are joined in order.  S = 1: one thread a pixel goes through all four; S = 4: each pixel has four threads
-// of the CTA (which takes 32 x 2 pixels), one a group.  The result is the same to the bit, and every choice within
-// it is the pixel's own: it depends neither on the crop nor on how many frames a launch has.
+// of the CTA (which takes 32 x 2 pixels), one a group; S = 0: one or the other, by how many pixels the mask has
+// gather.  The result is the same to the bit, and every choice within it is the pixel's own: it depends neither on the
+// crop nor on how many frames a launch has.
 template <int CFMT, bool DEBUG, bool SR, int INP, int S, bool LONG>
-__global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const GatherArgs a) {
-    static_assert(S == 1 || S == 4, "one thread a pixel or one a group");
-    constexpr int kRows = kFrTileY / S;
+__global__ void __launch_bounds__(kFrThreads, (kFrCtas<INP, LONG>)) frustum_kernel(const GatherArgs a) {
+    static_assert(S == 1 || S == 4 || (S == 0 && INP), "one thread a pixel, one a group, or (inpainting) as the mask has it");
     extern __shared__ float4 s_slot[];
     __shared__ float s_const[8];
     __shared__ unsigned long long s_cnt[2][kFrThreads / 32];
     __shared__ float s_w[kFrThreads / 32];
-    __shared__ FrSums s_red[S][kRows * 32];  // S = 1: the sums of the groups so far (in registers they spill)
-    __shared__ int s_dbg[DEBUG && S > 1 ? kRows * 32 : 1][2];
+    __shared__ FrSums s_red[kFrThreads];  // one thread a pixel: the sums of the groups so far (in registers they spill)
+    __shared__ int s_dbg[DEBUG && S != 1 ? kFrThreads : 1][2];
     const Planes &P = a.clip;
     const int oi = blockIdx.z;
     const int O = a.frame_begin + oi;
     const int ns = a.n_slots;
+    const int u = a.x0 + blockIdx.x * kFrTileX + threadIdx.x % kFrTileX;
+    int shares = S;  // threads a pixel
+    bool masked = false;
+    if (S == 0) {
+        // The mask at 16 x 16 places of the crop tells how many pixels gather.  The grid has a CTA for every 32 x 2
+        // pixels; with one thread a pixel the first quarter of them take 32 x 8.
+        const int su = a.x0 + (int)((2 * (threadIdx.x & 15) + 1) * (long long)a.cw / 32);
+        const int sv = a.y0 + (int)((2 * (threadIdx.x >> 4) + 1) * (long long)a.ch / 32);
+        const unsigned char *mp = P.mask + (long long)O * P.fstride + (long long)kPad * P.pitch + kPad;
+        const bool here = __ldg(mp + (long long)sv * P.pitch + su) != 0;
+        const int v4 = a.y0 + blockIdx.y * 2 + threadIdx.x / 32 % 2;
+        if (u < a.x0 + a.cw && v4 < a.y0 + a.ch) masked = __ldg(mp + (long long)v4 * P.pitch + u) != 0;
+        const long long n = (long long)__syncthreads_count(here) * a.cw * a.ch / 65536 * a.n_out;  // CTAs' worth of pixels
+        shares = frustum_shares(n, (long long)kFrCtas<INP, LONG> * a.sms, ns) ? 4 : 1;
+        if (shares == 1 && (int)blockIdx.y >= (a.ch + kFrTileY - 1) / kFrTileY) return;
+    }
+    const int rows = kFrTileY / shares;
+    const int Wo = SR ? P.W * a.sr_scale : P.W;
+    const int Ho = SR ? P.H * a.sr_scale : P.H;
+
+    const int lane = threadIdx.x % kFrTileX, row = threadIdx.x / kFrTileX % rows, split = threadIdx.x / (kFrTileX * rows);
+    const int v = a.y0 + blockIdx.y * rows + row;
+    const bool active = u < a.x0 + a.cw && v < a.y0 + a.ch;
+    const long long crop_idx = (long long)(v - a.y0) * a.cw + (u - a.x0);
+    const float L = 0.5f * a.frustum_l, nearp = a.near_plane, farp = a.far_plane;
+    const float zmid = 0.5f * (nearp + farp), zhalf = 0.5f * (farp - nearp);
+
+    float3 cref = make_float3(0.f, 0.f, 0.f);
+    float dref = 0.0f;
+    if (active && !SR) {
+        const long long pix = (long long)O * P.fstride + (long long)(v + kPad) * P.pitch + (u + kPad);
+        dref = __ldg(P.depth + pix);
+        cref = load_colour<CFMT>(P.colour, pix);
+    }
+    if (active && SR) {
+        // bilinear s_ref at input coordinates ((u, v) + 0.5) / scale - 0.5, clamped to the image; an
+        // invalid (NaN) depth among the four propagates and invalidates the reference
+        const float is = 1.0f / (float)a.sr_scale;
+        const float xc = fminf(fmaxf(((float)u + 0.5f) * is - 0.5f, 0.0f), (float)(P.W - 1));
+        const float yc = fminf(fmaxf(((float)v + 0.5f) * is - 0.5f, 0.0f), (float)(P.H - 1));
+        const int x0 = (int)floorf(xc), y0 = (int)floorf(yc);
+        const int x1 = min(x0 + 1, P.W - 1), y1 = min(y0 + 1, P.H - 1);
+        const float fx = xc - (float)x0, fy = yc - (float)y0;
+        const long long fb = (long long)O * P.fstride;
+        const long long p00 = fb + (long long)(y0 + kPad) * P.pitch + (x0 + kPad), p10 = p00 + (x1 - x0);
+        const long long p01 = fb + (long long)(y1 + kPad) * P.pitch + (x0 + kPad), p11 = p01 + (x1 - x0);
+        const float3 c00 = load_colour<CFMT>(P.colour, p00), c10 = load_colour<CFMT>(P.colour, p10);
+        const float3 c01 = load_colour<CFMT>(P.colour, p01), c11 = load_colour<CFMT>(P.colour, p11);
+        const float d00 = __ldg(P.depth + p00), d10 = __ldg(P.depth + p10), d01 = __ldg(P.depth + p01),
+                    d11 = __ldg(P.depth + p11);
+        const float gx = 1.0f - fx, gy = 1.0f - fy;
+        cref.x = gy * (gx * c00.x + fx * c10.x) + fy * (gx * c01.x + fx * c11.x);
+        cref.y = gy * (gx * c00.y + fx * c10.y) + fy * (gx * c01.y + fx * c11.y);
+        cref.z = gy * (gx * c00.z + fx * c10.z) + fy * (gx * c01.z + fx * c11.z);
+        dref = gy * (gx * d00 + fx * d10) + fy * (gx * d01 + fx * d11);
+    }
+    // inpainting gathers for masked pixels only and does not need their depth; the others need
+    // a valid reference depth (NaN fails)
+    const long long pix_o = (long long)O * P.fstride + (long long)(v + kPad) * P.pitch + (u + kPad);
+    if (INP && shares == 1) masked = active && __ldg(P.mask + pix_o) != 0;
+    const bool gather = INP ? masked : active && dref > 0.0f;
+    if (INP && active) cref = load_colour<CFMT>(P.colour, pix_o);
+    if (INP && !DEBUG && !__syncthreads_or(gather)) {
+        // no pixel of the CTA gathers: the output is the input
+        if (active && split == 0) {
+            float *o = P.out + (((long long)O * P.H + v) * P.W + u) * 3;
+            o[0] = cref.x;
+            o[1] = cref.y;
+            o[2] = cref.z;
+        }
+        return;
+    }
     for (int j = threadIdx.x; j < ns; j += kFrThreads) {
         const PairGeom &gf = a.geom[(long long)oi * ns + j], &gb = a.geom_back[(long long)oi * ns + j];
         float4 *d = s_slot + kFrSlotVec * j;
@@ -278,55 +351,10 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
         s_const[6] = gO.cx;
         s_const[7] = gO.cy;
     }
-    if (DEBUG && S > 1 && threadIdx.x < kRows * 32) s_dbg[threadIdx.x][0] = s_dbg[threadIdx.x][1] = 0;
+    if (DEBUG && S != 1) s_dbg[threadIdx.x][0] = s_dbg[threadIdx.x][1] = 0;
     __syncthreads();
     const float a_rgb = s_const[0], a_xyz = s_const[1], a_area = SR ? s_const[3] : 0.0f;
     const bool weighted = s_const[2] != 0.0f;
-    const int Wo = SR ? P.W * a.sr_scale : P.W;
-    const int Ho = SR ? P.H * a.sr_scale : P.H;
-
-    const int lane = threadIdx.x % kFrTileX, row = threadIdx.x / kFrTileX % kRows, split = threadIdx.x / (kFrTileX * kRows);
-    const int u = a.x0 + blockIdx.x * kFrTileX + lane;
-    const int v = a.y0 + blockIdx.y * kRows + row;
-    const bool active = u < a.x0 + a.cw && v < a.y0 + a.ch;
-    const long long crop_idx = (long long)(v - a.y0) * a.cw + (u - a.x0);
-    const float L = 0.5f * a.frustum_l, nearp = a.near_plane, farp = a.far_plane;
-    const float zmid = 0.5f * (nearp + farp), zhalf = 0.5f * (farp - nearp);
-
-    float3 cref = make_float3(0.f, 0.f, 0.f);
-    float dref = 0.0f;
-    if (active && !SR) {
-        const long long pix = (long long)O * P.fstride + (long long)(v + kPad) * P.pitch + (u + kPad);
-        dref = __ldg(P.depth + pix);
-        cref = load_colour<CFMT>(P.colour, pix);
-    }
-    if (active && SR) {
-        // bilinear s_ref at input coordinates ((u, v) + 0.5) / scale - 0.5, clamped to the image; an
-        // invalid (NaN) depth among the four propagates and invalidates the reference
-        const float is = 1.0f / (float)a.sr_scale;
-        const float xc = fminf(fmaxf(((float)u + 0.5f) * is - 0.5f, 0.0f), (float)(P.W - 1));
-        const float yc = fminf(fmaxf(((float)v + 0.5f) * is - 0.5f, 0.0f), (float)(P.H - 1));
-        const int x0 = (int)floorf(xc), y0 = (int)floorf(yc);
-        const int x1 = min(x0 + 1, P.W - 1), y1 = min(y0 + 1, P.H - 1);
-        const float fx = xc - (float)x0, fy = yc - (float)y0;
-        const long long fb = (long long)O * P.fstride;
-        const long long p00 = fb + (long long)(y0 + kPad) * P.pitch + (x0 + kPad), p10 = p00 + (x1 - x0);
-        const long long p01 = fb + (long long)(y1 + kPad) * P.pitch + (x0 + kPad), p11 = p01 + (x1 - x0);
-        const float3 c00 = load_colour<CFMT>(P.colour, p00), c10 = load_colour<CFMT>(P.colour, p10);
-        const float3 c01 = load_colour<CFMT>(P.colour, p01), c11 = load_colour<CFMT>(P.colour, p11);
-        const float d00 = __ldg(P.depth + p00), d10 = __ldg(P.depth + p10), d01 = __ldg(P.depth + p01),
-                    d11 = __ldg(P.depth + p11);
-        const float gx = 1.0f - fx, gy = 1.0f - fy;
-        cref.x = gy * (gx * c00.x + fx * c10.x) + fy * (gx * c01.x + fx * c11.x);
-        cref.y = gy * (gx * c00.y + fx * c10.y) + fy * (gx * c01.y + fx * c11.y);
-        cref.z = gy * (gx * c00.z + fx * c10.z) + fy * (gx * c01.z + fx * c11.z);
-        dref = gy * (gx * d00 + fx * d10) + fy * (gx * d01 + fx * d11);
-    }
-    // inpainting gathers for masked pixels only and does not need their depth; the others need
-    // a valid reference depth (NaN fails)
-    const long long pix_o = (long long)O * P.fstride + (long long)(v + kPad) * P.pitch + (u + kPad);
-    const bool gather = INP ? active && __ldg(P.mask + pix_o) != 0 : active && dref > 0.0f;
-    if (INP && active) cref = load_colour<CFMT>(P.colour, pix_o);
     // semi-transparency: the pixel's own sample (I(p), x_ref, O) needs a valid depth (NaN fails)
     const float3 c_in = cref;
     const bool own = INP == 2 && dref > 0.0f;
@@ -339,7 +367,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
     long long n_exam = 0;
     int n_acc = 0;
     if (DEBUG && active && !gather && a.membership)
-        for (int j = split; j < ns; j += S) {
+        for (int j = split; j < ns; j += shares) {
             int32_t *rec = a.membership + (crop_idx * ns + j) * 4;
             rec[0] = -2; rec[1] = 0; rec[2] = 0; rec[3] = 0;
         }
@@ -351,7 +379,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
     m_log2 = wpass ? kNoWeight : 0.0f;
     if (gather) {
       bool first = true;
-      for (int grp = split; grp < 4; grp += S) {
+      for (int grp = split; grp < 4; grp += shares) {
         const int j0 = (grp - (O - a.T)) & 3;
         if (j0 >= ns) continue;  // joining an empty group's zeros changes nothing
         for (int j = j0; j < ns; j += 4) {
@@ -739,8 +767,8 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
                 rec[3] = (int32_t)(unsigned int)(mh >> 32);
             }
         }
-        if (S == 1 && ns > 1) {
-            FrSums part = {acc_r, acc_g, acc_b, acc_w, m_log2}, &sum = s_red[0][threadIdx.x];
+        if (shares == 1 && ns > 1) {
+            FrSums part = {acc_r, acc_g, acc_b, acc_w, m_log2}, &sum = s_red[threadIdx.x];
             if (!first) {
                 FrSums all = sum;
                 join_sums(all, part);
@@ -752,8 +780,8 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
             m_log2 = wpass ? kNoWeight : 0.0f;
         }
       }
-      if (S == 1 && ns > 1) {
-          const FrSums sum = s_red[0][threadIdx.x];
+      if (shares == 1 && ns > 1) {
+          const FrSums sum = s_red[threadIdx.x];
           acc_r = sum.r;
           acc_g = sum.g;
           acc_b = sum.b;
@@ -761,14 +789,14 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
           m_log2 = sum.m;
       }
     }
-    if (S > 1) {
+    if (shares > 1) {
         // join the four threads' sums; every thread takes the result
         const int px = row * 32 + lane;
-        s_red[split][px] = {acc_r, acc_g, acc_b, acc_w, m_log2};
+        s_red[threadIdx.x] = {acc_r, acc_g, acc_b, acc_w, m_log2};
         __syncthreads();
-        FrSums sum = s_red[0][px];
+        FrSums sum = s_red[px];
 #pragma unroll
-        for (int s = 1; s < S; ++s) join_sums(sum, s_red[s][px]);
+        for (int s = 1; s < 4; ++s) join_sums(sum, s_red[s * (kFrThreads / 4) + px]);
         acc_r = sum.r;
         acc_g = sum.g;
         acc_b = sum.b;
@@ -787,7 +815,7 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
     }
     }  // passes
 
-    if (DEBUG && S > 1) {
+    if (DEBUG && S != 1) {
         atomicAdd(&s_dbg[row * 32 + lane][0], n_acc);
         atomicAdd(&s_dbg[row * 32 + lane][1], (int)min(n_exam, 0x7fffffffll));
         __syncthreads();
@@ -806,8 +834,8 @@ __global__ void __launch_bounds__(kFrThreads, kFrCtas<INP>) frustum_kernel(const
         o[2] = o_b;
         if (DEBUG && a.pixel_stats) {
             int32_t *ps = a.pixel_stats + crop_idx * 3;
-            ps[0] = S > 1 ? s_dbg[row * 32 + lane][0] : n_acc;
-            ps[1] = S > 1 ? s_dbg[row * 32 + lane][1] : (int32_t)min(n_exam, 0x7fffffffll);
+            ps[0] = S != 1 ? s_dbg[row * 32 + lane][0] : n_acc;
+            ps[1] = S != 1 ? s_dbg[row * 32 + lane][1] : (int32_t)min(n_exam, 0x7fffffffll);
             ps[2] = __float_as_int(sw_true);
         }
     }
@@ -874,7 +902,7 @@ __global__ void __launch_bounds__(256) zrange_kernel(Planes P, unsigned int *zr,
 
 template <bool SR, int INP, int S, bool LONG>
 cudaError_t launch_frustum_t(const GatherArgs &a, cudaStream_t s) {
-    constexpr int kRows = kFrTileY / S;
+    constexpr int kRows = kFrTileY / (S == 1 ? 1 : 4);
     const dim3 grid((a.cw + kFrTileX - 1) / kFrTileX, (a.ch + kRows - 1) / kRows, a.n_out);
     const bool dbg = a.membership || a.pixel_stats;
     const size_t smem = sizeof(float4) * kFrSlotVec * (size_t)a.n_slots;  // at most 32 KB
@@ -925,16 +953,18 @@ __global__ void __launch_bounds__(256) mask_box_kernel(Planes P, const double *c
 
 }  // namespace
 
-// Four threads a pixel for inpainting and semi-transparency, which gather for few of the frame's pixels, in three
-// passes (720p, one box removed: 1.19 ms with one thread a pixel, 0.42 with four, 0.49 with eight).
-cudaError_t launch_frustum(const GatherArgs &a, cudaStream_t s) {
-    if (a.mode == SSVP_MODE_INPAINT && !a.sr_out) return launch_frustum_s<false, 1, 4>(a, s);
-    if (a.mode == SSVP_MODE_SEMI && !a.sr_out) return launch_frustum_s<false, 2, 4>(a, s);
+// Inpainting and semi-transparency gather for the masked pixels alone, in three passes; how many there are is known on
+// the device only, so that a CTA decides itself.
+cudaError_t launch_frustum(const GatherArgs &args, cudaStream_t s) {
+    GatherArgs a = args;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    a.sms = sms;
+    if (a.mode == SSVP_MODE_INPAINT && !a.sr_out) return launch_frustum_s<false, 1, 0>(a, s);
+    if (a.mode == SSVP_MODE_SEMI && !a.sr_out) return launch_frustum_s<false, 2, 0>(a, s);
     const long long ctas = (long long)((a.cw + kFrTileX - 1) / kFrTileX) * ((a.ch + kFrTileY - 1) / kFrTileY) * a.n_out;
-    const bool shared = frustum_shares(ctas, kFrCtas<0> * sms, a.n_slots);
+    const bool shared = frustum_shares(ctas, 3ll * sms, a.n_slots);
     if (a.sr_out) return shared ? launch_frustum_s<true, 0, 4>(a, s) : launch_frustum_s<true, 0, 1>(a, s);
     return shared ? launch_frustum_s<false, 0, 4>(a, s) : launch_frustum_s<false, 0, 1>(a, s);
 }

@@ -98,6 +98,7 @@ struct GatherArgs {
     // 2 as 1 but issues no copies, so that the waits run out (a test of the time-out path)
     int stage;
     int *err;                 // error word: bit 1 set when a staging wait timed out
+    int sms;                  // frustum gather: SMs of the device (set by its launch)
 };
 
 // One clip of a batched launch (A10).  Work items are (clip, output-frame chunk, tile) triples

@@ -37,4 +37,14 @@ SSVP_HD inline bool frustum_shares(long long ctas, long long wave, int n_slots) 
     return (n_slots >= 3 && 4 * ctas <= wave) || (n_slots >= 5 && 5 * ctas <= 3 * wave) || (n_slots >= 7 && 2 * ctas < 3 * wave);
 }
 
+// Window gather, us with one thread and with four (k = 7, and k = 3 where named): 96 x 54 (0.03 waves) 0 13.5, 13.4, +-1
+// 17.3, 13.4; 320 x 180 (0.4) 0 16.9, 19.6, +-1 23.6, 21.2, +-15 120, 71; 480 x 270 (0.8) 0 21.8, 31.2, +-2 42.9, 45.7,
+// +-3 51.9, 51.3, k = 3 +-2 28.7, 34.0; 560 x 316 (1.2) +-2 59.4, 57.7, +-3 75.8, 64.3, +-5 108, 85, k = 3 +-5 53.7,
+// 51.8; 640 x 360 (1.5) +-2 60.3, 65.4, +-3 79.1, 75.1, +-15 321, 262, k = 3 +-5 54.6, 58.4, +-15 147, 133; 853 x 479
+// (2.7) +-8 284, 284, k = 3 135, 151; 720p (5.9) +-15 949, 986
+SSVP_HD inline bool window_shares(long long ctas, long long wave, int n_slots, int k) {
+    return (n_slots >= 3 && 2 * ctas <= wave) || (n_slots >= 7 && ctas < wave) || (n_slots >= 7 && n_slots * k >= 49 && 2 * ctas < 3 * wave) ||
+           (n_slots >= 16 && 2 * ctas < 5 * wave);
+}
+
 }  // namespace ssvp

@@ -36,6 +36,7 @@
 
 #include "../../include/ssvp.h"
 #include "ssvp_df.cuh"
+#include "ssvp_dispatch.h"
 #include "ssvp_internal.h"
 
 namespace ssvp {
@@ -1208,17 +1209,12 @@ cudaError_t launch_k(const GatherArgs &a, cudaStream_t s) {
     else if (a.sets.col) gather_kernel<K, CFMT, false, 1, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
     else if (dbg) gather_kernel<K, CFMT, true><<<grid, kThreads, smem, s>>>(a, tmap);
     else {
-        // Few CTAs leave SMs idle or end in a nearly empty wave: below two and a half waves each pixel's frames
-        // are shared out to four threads (CTAs of 32 x 2 pixels).  One frame of 320 x 180, +-15 (0.4 waves):
-        // 104 -> 73 us; the 16 frames of 160 x 90 (1.6): 100 -> 96; 640 x 360 (1.5): 312 -> 261; six frames of
-        // 320 x 180 (2.3): 300 -> 275; two of 640 x 360, k = 5 (3.0): 351 against 360, one of 720p (5.9) 940 against 976.
-        // Each CTA builds the geometry of all frames, so above one wave only for windows of 16 frames and more
-        // (669 x 379, +-3, k = 3, 1.7 waves: 2 % slower shared out).
+        // Few CTAs leave SMs idle or end in a nearly empty wave: then each pixel's frames are shared out to four
+        // threads (CTAs of 32 x 2 pixels)
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const long long ctas = (long long)grid.x * grid.y * grid.z, wave = (long long)SSVP_MIN_CTAS * sms;
-        if (ctas < wave || (2 * ctas < 5 * wave && a.n_slots >= 16)) {
+        if (window_shares((long long)grid.x * grid.y * grid.z, (long long)SSVP_MIN_CTAS * sms, a.n_slots, a.k)) {
             grid.y = (a.ch + kTileY / 4 - 1) / (kTileY / 4);
             gather_kernel<K, CFMT, false, false, SSVP_MIN_CTAS, false, 4><<<grid, kThreads, smem, s>>>(a, tmap);
         } else gather_kernel<K, CFMT, false><<<grid, kThreads, smem, s>>>(a, tmap);

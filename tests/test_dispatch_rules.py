@@ -51,3 +51,14 @@ def test_frustum_frames_shared(rule):
     no = [(96, 54, 0), (320, 180, 0), (320, 180, 1), (480, 270, 0), (480, 270, 2), (640, 360, 3), (640, 360, 15), (1280, 720, 30)]
     assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
     assert rule(*(call(*c) for c in no)) == [0] * len(no)
+
+
+def test_window_frames_shared(rule):
+    def call(W, H, T, k, n=1):
+        return f"window_shares({ctas(W, H, n)}, {4 * SMS}, {2 * T + 1}, {k})"
+    yes = [(96, 54, 1, 7), (320, 180, 1, 7), (320, 180, 15, 3), (480, 270, 3, 7), (560, 316, 5, 7), (640, 360, 3, 7), (640, 360, 15, 3), (160, 90, 15, 5, 16),
+           (320, 180, 15, 7, 6)]
+    no = [(96, 54, 0, 7), (320, 180, 0, 3), (480, 270, 0, 7), (480, 270, 1, 3), (480, 270, 2, 7), (560, 316, 1, 7), (640, 360, 2, 7), (640, 360, 5, 3),
+          (853, 479, 5, 7), (853, 479, 15, 7), (1280, 720, 30, 7)]
+    assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
+    assert rule(*(call(*c) for c in no)) == [0] * len(no)

@@ -23,6 +23,7 @@
 #include <cuda_fp16.h>
 
 #include "ssvp_df.cuh"
+#include "ssvp_dispatch.h"
 #include "ssvp_internal.h"
 
 namespace ssvp {
@@ -349,8 +350,6 @@ cudaError_t launch_aperture_t(const GatherArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Four threads a pixel where one gives less than three waves of CTAs: FP16 colour, 480 x 270, +-30 (1.1 waves) 1.65 ->
-// 1.21 ms, 640 x 360, +-15 (2.0) 1.25 -> 1.10, FP32 (1.5) 1.54 -> 1.16; 1080p, +-10 (18) 11.2 against 11.5
 template <int CFMT>
 cudaError_t launch_aperture_c(const GatherArgs &a, cudaStream_t s) {
     if (a.membership || a.pixel_stats) return launch_aperture_t<CFMT, true, 1>(a, s);
@@ -358,7 +357,7 @@ cudaError_t launch_aperture_c(const GatherArgs &a, cudaStream_t s) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const long long ctas = (long long)((a.cw + 31) / 32) * ((a.ch + kApTileY - 1) / kApTileY) * a.n_out;
-    return ctas < 3ll * kApCtas<CFMT> * sms ? launch_aperture_t<CFMT, false, 4>(a, s) : launch_aperture_t<CFMT, false, 1>(a, s);
+    return aperture_shares(ctas, (long long)kApCtas<CFMT> * sms, a.n_slots) ? launch_aperture_t<CFMT, false, 4>(a, s) : launch_aperture_t<CFMT, false, 1>(a, s);
 }
 }  // namespace
 

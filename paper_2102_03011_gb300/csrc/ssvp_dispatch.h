@@ -47,4 +47,13 @@ SSVP_HD inline bool window_shares(long long ctas, long long wave, int n_slots, i
            (n_slots >= 16 && 2 * ctas < 5 * wave);
 }
 
+// Virtual aperture, us with one thread and with four (FP32 colour): 320 x 180 (0.4 waves) 0 29.9, 41.3, +-1 62.9, 48.7,
+// +-2 95, 79; 640 x 360 (1.5) 0 64.4, 119, +-1 157, 147, +-2 249, 251, +-3 344, 285, +-15 1543, 1153; 853 x 479 (2.7) 0 110,
+// 223, +-1 268, 274, +-2 426, 463, +-3 602, 551, +-15 2616, 2190; FP16: 853 x 479 (3.6) +-2 390, 441, +-15 2441, 2096.
+// Where the chip is full already the frames have to divide well: five leave three of four threads idle half the time.
+SSVP_HD inline bool aperture_shares(long long ctas, long long wave, int n_slots) {
+    const int full = 4 * ((n_slots + 3) / 4);
+    return n_slots >= 3 && (ctas <= wave || (ctas < 3 * wave && 3 * n_slots >= 2 * full));
+}
+
 }  // namespace ssvp

@@ -62,3 +62,12 @@ def test_window_frames_shared(rule):
           (853, 479, 5, 7), (853, 479, 15, 7), (1280, 720, 30, 7)]
     assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
     assert rule(*(call(*c) for c in no)) == [0] * len(no)
+
+
+def test_aperture_frames_shared(rule):
+    def call(W, H, T, ctas_per_sm=4):
+        return f"aperture_shares({ctas(W, H)}, {ctas_per_sm * SMS}, {2 * T + 1})"
+    yes = [(96, 54, 1), (320, 180, 1), (320, 180, 2), (480, 270, 2), (640, 360, 1), (640, 360, 3), (853, 479, 15), (640, 360, 3, 3)]
+    no = [(96, 54, 0), (320, 180, 0), (640, 360, 0), (640, 360, 2), (853, 479, 2), (853, 479, 15, 3), (1280, 720, 15)]
+    assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
+    assert rule(*(call(*c) for c in no)) == [0] * len(no)

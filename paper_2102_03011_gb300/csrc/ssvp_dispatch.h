@@ -56,4 +56,8 @@ SSVP_HD inline bool aperture_shares(long long ctas, long long wave, int n_slots)
     return n_slots >= 3 && (ctas <= wave || (ctas < 3 * wave && 3 * n_slots >= 2 * full));
 }
 
+// Extraction of the learned filter's sets: four CTAs an SM where that is one wave and three an SM are not (figures at
+// kLearnCtas)
+SSVP_HD inline bool extract_four_ctas(long long ctas, int sms) { return ctas > 3ll * sms && ctas <= 4ll * sms; }
+
 }  // namespace ssvp

@@ -45,10 +45,11 @@ namespace {
 #ifndef SSVP_MIN_CTAS
 #define SSVP_MIN_CTAS 4  // resident CTAs per SM the register allocation must allow
 #endif
-// The extraction gather of the learned filter keeps more values live than the plain one: at 64 registers
-// (four CTAs per SM) it spills 96 bytes a thread, at 80 (three CTAs) none.  The gradient of a 16,384-pixel
-// batch of a 640 x 360 frame, +-15: 0.665 against 0.574 ms; a learned 1080p frame at +-30: 7.83 against
-// 7.77 ms, at +-6 3.96 against 3.96 ms.
+// The extraction gather of the learned filter keeps more values live than the plain one: at 64 registers (four CTAs
+// per SM) it spills 96 bytes a thread, at 80 (three CTAs) none.  640 x 360 (two waves of three), +-10: 531 against 508
+// us a learned frame; but where four CTAs an SM hold the whole launch in one wave and three do not, four are better:
+// 480 x 270, +-6, +-10 and +-15, 245, 312 and 374 against 257, 333 and 402 us; 532 x 293, a little more than one wave
+// of four, +-10, 394 against 383.
 constexpr int kLearnCtas = 3;
 
 #ifndef SSVP_TILE_Y
@@ -1206,8 +1207,13 @@ cudaError_t launch_k(const GatherArgs &a, cudaStream_t s) {
     // 1.30 -> 1.27, 640 x 360 0.80 -> 0.82, 480 x 270 0.51 -> 0.52
     if (a.sets.col && (long long)a.cw * a.ch >= 300000)
         gather_kernel<K, CFMT, false, 2, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
-    else if (a.sets.col) gather_kernel<K, CFMT, false, 1, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
-    else if (dbg) gather_kernel<K, CFMT, true><<<grid, kThreads, smem, s>>>(a, tmap);
+    else if (a.sets.col) {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        if (extract_four_ctas((long long)grid.x * grid.y * grid.z, sms)) gather_kernel<K, CFMT, false, 1, kLearnCtas + 1><<<grid, kThreads, smem, s>>>(a, tmap);
+        else gather_kernel<K, CFMT, false, 1, kLearnCtas><<<grid, kThreads, smem, s>>>(a, tmap);
+    } else if (dbg) gather_kernel<K, CFMT, true><<<grid, kThreads, smem, s>>>(a, tmap);
     else {
         // Few CTAs leave SMs idle or end in a nearly empty wave: then each pixel's frames are shared out to four
         // threads (CTAs of 32 x 2 pixels)

@@ -71,3 +71,8 @@ def test_aperture_frames_shared(rule):
     no = [(96, 54, 0), (320, 180, 0), (640, 360, 0), (640, 360, 2), (853, 479, 2), (853, 479, 15, 3), (1280, 720, 15)]
     assert rule(*(call(*c) for c in yes)) == [1] * len(yes)
     assert rule(*(call(*c) for c in no)) == [0] * len(no)
+
+
+def test_extraction_ctas(rule):
+    sizes = [(160, 90), (320, 180), (480, 270), (532, 293), (640, 360), (1920, 1080)]
+    assert rule(*(f"extract_four_ctas({ctas(*s)}, {SMS})" for s in sizes)) == [0, 0, 1, 0, 0, 0]

@@ -530,7 +530,8 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
             const float dj_t = LEARN ? (float)(j - Tw) * inv_T : 0.0f;  // the frame-offset feature
             if (DEBUG && rec) {
                 rec[0] = 1; rec[1] = cx; rec[2] = cy;
-                for (int wd = 3; wd < rec_words; ++wd) rec[wd] = 0;
+                if (K == 0)
+                    for (int wd = 3; wd < rec_words; ++wd) rec[wd] = 0;
             }
             // The depth test |d_q - z'| < r is necessary for the radius test (d^2 >= dz^2 in FP32 too: the
             // other terms are added to it).  It is evaluated as e^2 < thr, e = d_q - zh without the low
@@ -611,7 +612,11 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
                         const float w = weighted ? ex2(e) : 1.0f;
                         if (ok[t] && d2 < r2) {
                             n_acc += 1.0f;
-                            if (DEBUG) acc_bits[(im[t] >> 5) & 1] |= 0x80000000u >> (im[t] & 31);
+                            if (DEBUG) {
+                                const unsigned bit = 0x80000000u >> (im[t] & 31);
+                                if (WB::kWords == 2 && (im[t] & 32u)) acc_bits[1] |= bit;
+                                else acc_bits[0] |= bit;
+                            }
                             if (!LEARN) {
                                 acc_r = fmaf(w, er, acc_r);
                                 acc_g = fmaf(w, eg, acc_g);
@@ -654,11 +659,17 @@ __device__ __forceinline__ void gather_pixel(const GatherArgs &a, const Planes &
                     acc_w += s_w[0] + s_w[1];
                 }
                 if (DEBUG && rec) {
-                    for (int i = 0; i < K * WB::kC; ++i)  // record layout: bit dy*k+dx
-                        if (acc_bits[i >> 5] << (i & 31) >> 31) {
-                            const int bit = i / WB::kC * K + i % WB::kC;
-                            rec[3 + (bit >> 5)] |= (int32_t)(1u << (bit & 31));
-                        }
+                    // record layout: bit dy * k + dx from the bottom
+                    unsigned words[2] = {0u, 0u};
+#pragma unroll
+                    for (int dy = 0; dy < K; ++dy) {
+                        const int first = dy % WB::kRows * WB::kC, at = dy * K;
+                        const unsigned row = __brev(acc_bits[dy / WB::kRows] << first) & ((1u << K) - 1u);
+                        words[at / 32] |= row << at % 32;
+                        if (at % 32 + K > 32) words[1] |= row >> (32 - at % 32);
+                    }
+                    rec[3] = (int32_t)words[0];
+                    if (K * K > 32) rec[4] = (int32_t)words[1];
                 }
             } else {
                 for (int dy = 0; dy < k; ++dy) {

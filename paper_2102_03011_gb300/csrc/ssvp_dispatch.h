@@ -12,7 +12,7 @@ namespace ssvp {
 
 // Whether a frustum gather takes the instance that can drop whole blocks of a long hull.  Hulls grow with the image
 // and with the distance of the window's frames, and only long ones gain; the instance without it spills next to
-// nothing (with it 230 to 260 bytes a thread).  band: the hull's width in input pixels; a band of one or two pixels has
+// nothing (with it 230 to 280 bytes a thread).  band: the hull's width in input pixels; a band of one or two pixels has
 // few candidates to drop, in a wide one few blocks can be dropped.  Both sides, in ms with and without:
 //   band 3     960 x 540 +-15 1.73, 1.73; 720p +-15 3.21, 3.44; 640 x 360 +-30 1.80, 1.94; 720p +-30 8.15, 11.2;
 //              1080p +-30 20.5, 33.6

@@ -1,5 +1,5 @@
 // ssvp_frustum.cu - the paper's frustum gather (Sec. "Sample Gathering", Eq. 1-2) fused with the
-// Eq. 3/4 filter.  One thread per output pixel, window frames in order.
+// Eq. 3/4 filter.  One thread per output pixel, or four that share its window frames.
 //
 // Per (pixel p, frame J):
 //   1. The frustum V of Eq. 1 (the l x l square around p swept over O depths [near, far]) is
@@ -19,12 +19,12 @@
 //   3. Samples are weighted by Eq. 4 around s_ref (times the per-frame factors of Eq. 5, or by
 //      Eq. 10's shutter function alone) and reduced by Eq. 3, as in the window gather.
 //
-// What bounds it: instruction issue (0.73 of the slots).  Of a 720p +-15 frame's 3.2 ms the candidates' tests
-// take a third, taking the samples (4.4 of 104 candidates a pixel and frame, a third of a warp's lanes at a
-// time) a third, the bound of the hull 0.4 ms, the block checks 0.5 ms.  Against one walk of every row: 720p +-15
-// 3.77 -> 3.23 ms, 1080p +-30 37.0 -> 20.5, super-resolution 640 x 360 to 1080p 7.7 -> 7.1 (short hulls: the
-// geometry read from shared memory), inpainting 1.11 -> 0.34 and a 320 x 180 frame 0.223 -> 0.156 (four
-// threads a pixel).
+// What bounds it: instruction issue (720p, +-15, ncu: 0.70 of the slots, 3.10e9 warp instructions, ALU pipe 50 %; DRAM
+// 524 MB).  Of that frame's 3.2 ms the candidates' tests take about a third, taking the samples (4.4 of 104 candidates
+// a pixel and frame, a third of a warp's lanes at a time) a third, the bound of the hull 0.4 ms, the block checks 0.5
+// ms.  Against one walk of every row: 720p +-15 3.76 -> 3.22 ms, 1080p +-30 36.9 -> 20.5, super-resolution 640 x 360 to
+// 1080p 7.70 -> 6.89 (short hulls: the geometry read from shared memory); with four threads a pixel a 320 x 180
+// frame 221 -> 146 us, inpainting of a 720p frame, one small box 1.06 -> 0.28 ms, a fifth of the frame 3.28 -> 3.11.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -172,7 +172,7 @@ __device__ __forceinline__ bool lateral_fast(const float (&Ma)[3], const float (
 }
 
 // Registers: 80 (three CTAs per SM), with some spilled in the form that can drop blocks.  For inpainting that form has 128
-// (two CTAs) instead: 720p, +-15, one box of 1 % of the frame, 331 against 354 us.  The other is better off with
+// (two CTAs) instead: 720p, +-15, one small box, 275 against 354 us.  The other is better off with
 // three CTAs, which spill nothing: 640 x 360, +-5, two fifths of the frame masked, 262 against 335 us.
 template <int INP, bool LONG> constexpr int kFrCtas = INP && LONG ? 2 : 3;
 constexpr int kFrSlotVec = 8;  // float4 words of a window slot in shared memory:

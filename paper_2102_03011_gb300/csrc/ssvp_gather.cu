@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(32 * TY, 32 / TY) batch_kernel(const GatherArg
 // then take each frame's window together, lane = candidate (rows 0-3, then 4-6 of an 8-column grid); the
 // accepted ones, in canonical order, queue up and are filtered 32 at a time.  The geometry is that of the tiles
 // of gather_kernel, so the sets are the same; the plain result's sums are per lane and differ in rounding.
-// Bound by instruction issue (0.70 of the slots): 4,200 warp instructions a pixel at +-15 (5,000 and 131
+// Bound by instruction issue (0.71 of the slots, ncu): 4,200 warp instructions a pixel at +-15 (5,000 and 131
 // instead of 105 us for 16,384 pixels with each window's few samples filtered at once).  Extracting the whole
 // 640 x 360 frame takes 385 us; the gradient of the batch went from 0.60 to 0.25 ms, with the training
 // kernel's operand layout.

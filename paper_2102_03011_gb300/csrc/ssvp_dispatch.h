@@ -12,8 +12,9 @@ namespace ssvp {
 
 // Whether a frustum gather takes the instance that can drop whole blocks of a long hull.  Hulls grow with the image
 // and with the distance of the window's frames, and only long ones gain; the instance without it spills next to
-// nothing (with it 230 to 280 bytes a thread).  band: the hull's width in input pixels; a band of one or two pixels has
-// few candidates to drop, in a wide one few blocks can be dropped.  Both sides, in ms with and without:
+// nothing (with it 230 to 280 bytes a thread).  side: the image's longer side; band: the hull's width in input pixels; a
+// band of one or two pixels has few candidates to drop, in a wide one few blocks can be dropped.  Both sides, in ms with
+// and without:
 //   band 3     960 x 540 +-15 1.73, 1.73; 720p +-15 3.21, 3.44; 640 x 360 +-30 1.80, 1.94; 720p +-30 8.15, 11.2;
 //              1080p +-30 20.5, 33.6
 //   band 9     640 x 360 +-30 6.71, 6.13; 1080p +-15 28.4, 29.9; 6: 720p +-15 6.77, 6.82
@@ -21,8 +22,8 @@ namespace ssvp {
 //   super-resolution: x 3 of 640 x 360, +-30 (band 0.3, 1) 6.18, 4.39 and 7.58, 6.89; x 2 of 720p, +-15 (0.5, 1.5) 5.93,
 //              4.51 and 7.82, 7.62, +-30 16.7, 14.8 and 20.2, 25.3; x 2 of 640 x 360, +-60 (1.5) 10.6, 13.2
 // A rule on the whole image and the window, not on the crop: the two sum in different orders.
-inline bool frustum_long_hulls(int n_slots, int width, float band) {
-    return (long long)n_slots * width >= (band < 1.0f ? 100000 : band < 2.0f ? 70000 : band < 5.0f ? 35000 : 50000);
+inline bool frustum_long_hulls(int n_slots, int side, float band) {
+    return (long long)n_slots * side >= (band < 1.0f ? 100000 : band < 2.0f ? 70000 : band < 5.0f ? 35000 : 50000);
 }
 
 // Whether each pixel's window frames are shared out to four threads, where one thread a pixel fills the chip badly.

@@ -915,7 +915,9 @@ cudaError_t launch_frustum_t(const GatherArgs &a, cudaStream_t s) {
 
 template <bool SR, int INP, int S>
 cudaError_t launch_frustum_s(const GatherArgs &a, cudaStream_t s) {
-    return frustum_long_hulls(a.n_slots, a.clip.W, SR ? a.frustum_l / (float)a.sr_scale : a.frustum_l) ? launch_frustum_t<SR, INP, S, true>(a, s) : launch_frustum_t<SR, INP, S, false>(a, s);
+    const float band = SR ? a.frustum_l / (float)a.sr_scale : a.frustum_l;
+    return frustum_long_hulls(a.n_slots, std::max(a.clip.W, a.clip.H), band) ? launch_frustum_t<SR, INP, S, true>(a, s)
+                                                                             : launch_frustum_t<SR, INP, S, false>(a, s);
 }
 
 // Eq. 8-9's mask from a scene-space box: per pixel of every frame, the world point of its depth
